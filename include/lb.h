@@ -88,9 +88,11 @@ typedef struct {
   int precision;          /* lb_precision */
   int nu_every;           /* > 0: accumulate Nu_mean every nu_every steps into the time average */
   int check_every;        /* > 0: lb_step checks rho > 0, T > 0, no NaN every check_every steps */
-  int tile_y;             /* launch shape: CTA tile is 32 x tile_y (4, 8 or 16; 16 not with FP64;
-                             0 = default: 8) */
-  int z_chunk;            /* launch shape: planes per CTA (0 = choose from the grid size) */
+  int tile_y;             /* launch shape of the tile march: CTA tile is 32 x tile_y (4, 8 or 16;
+                             16 not with FP64; 0 = 8) */
+  int z_chunk;            /* launch shape of the tile march: planes per CTA (0 = choose from the
+                             grid size). With tile_y = z_chunk = 0 the library chooses the form
+                             of the step as well: see lb_step */
   int forcing;            /* LB_FORCE_SHIFT (0, the paper) or LB_FORCE_GUO */
   int psi_kind;           /* LB_PSI_EXP (0, the paper) or LB_PSI_VDW */
   double vdw_a, vdw_b;    /* LB_PSI_VDW: attraction a > 0 and excluded volume b > 0 */
@@ -111,8 +113,11 @@ typedef struct lb_ctx lb_ctx;  /* opaque */
 int lb_init(const lb_params* params, const double* rho_init, const double* T_init,
             int init_on_device, void* cuda_stream, lb_ctx** out);
 
-/* lb_step -- advance nsteps time steps of Eqs. (6)-(7): per step one fused launch that pull-
- * streams f and g (periodic x/y, bounce-back walls), takes the moments of Eq. (8), the force of
+/* lb_step -- advance nsteps time steps of Eqs. (6)-(7). A context with a launch shape (tile_y or
+ * z_chunk) takes the tile march: per step one fused launch (FP64: after a pass that forms the moments
+ * of every node). Otherwise the library chooses by precision and grid size between a march in one
+ * launch with separate warps for the moments and the collision, and three streaming kernels
+ * (moments, velocities, collision); the forms differ in rounding only. A step pull-streams f and g (periodic x/y, bounce-back walls), takes the moments of Eq. (8), the force of
  * Eq. (9) with psi = exp(-1/rho) plus gravity rho g_z z (psi_kind selects the variant), the shifted
  * velocity u' = (j + tau_nu F)/rho (forcing selects the variant),
  * the physical velocity u = (j + F/2)/rho and its divergence, and collides f (temperature in
@@ -229,8 +234,9 @@ int lb_load(lb_ctx* ctx, const char* path);
 /* lb_step_count -- number of steps taken since lb_init (or restored by lb_load); -1 if ctx is NULL. */
 long long lb_step_count(const lb_ctx* ctx);
 
-/* lb_launch_info -- how the context's step kernel is launched (launch metadata for performance
- * reports; the paper has no counterpart). Host output of 6 ints: out[0], out[1] = grid (column
+/* lb_launch_info -- the launch shape of the context's tile march, the step kernel of a context with
+ * tile_y or z_chunk set (a context that leaves both 0 steps with the form that lb_step describes);
+ * launch metadata for performance reports, the paper has no counterpart. Host output of 6 ints: out[0], out[1] = grid (column
  * tiles, z chunks), out[2] = threads per CTA, out[3] = dynamic shared memory bytes per CTA,
  * out[4] = CTAs resident per SM as the CUDA occupancy calculator reports it, out[5] = registers
  * per thread. Errors: LB_EINVAL (NULL argument), LB_ECUDA. */

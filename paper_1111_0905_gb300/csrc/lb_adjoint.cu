@@ -368,6 +368,17 @@ using namespace tlbm;
 
 namespace {
 
+// The step of state n writes the fields that the reverse sweep reads straight into m
+// ([MF_COUNT][N]): the three-kernel step keeps its own fields there.
+void adj_fields(KArgs& a, double* m) {
+  a.adj_m = m;
+  if (!a.fd_rho) return;
+  const size_t N = (size_t)a.N;
+  a.fd_rho = m + MF_RHO * N;
+  a.fd_psi = m + MF_PSI * N;
+  for (int k = 0; k < 3; ++k) { a.fd_u[k] = m + (MF_UX + k) * N; a.fd_v[k] = m + (MF_VX + k) * N; }
+}
+
 struct DevBuf {
   void* p = nullptr;
   ~DevBuf() { if (p) cudaFree(p); }
@@ -454,7 +465,6 @@ extern "C" int lb_adjoint_step(lb_ctx* c, long long nsteps, int checkpoint_every
   };
 
   // forward: checkpoints every K steps; with FP64 storage the last segment's fields as it goes
-  const dim3 grid = fused_grid(c);
   const long long n0_last = (nck - 1) * K;
   for (long long n = 0; n < nsteps; ++n) {
     if (n % K == 0) {
@@ -463,8 +473,8 @@ extern "C" int lb_adjoint_step(lb_ctx* c, long long nsteps, int checkpoint_every
       LB_CU(c, cudaMemcpyAsync(dst + pbytes, c->g[c->cur], pbytes, cudaMemcpyDeviceToDevice, st));
     }
     KArgs a = make_args(c);
-    if (fields && n >= n0_last) a.adj_m = Ms + (size_t)(n - n0_last) * mstate;
-    LB_CU(c, c->ops->fused(a, MODE_STEP, c->by, grid, st));
+    if (fields && n >= n0_last) adj_fields(a, Ms + (size_t)(n - n0_last) * mstate);
+    LB_CU(c, launch_step(c, a, MODE_STEP));
     c->cur ^= 1;
     c->step += 1;
   }
@@ -493,12 +503,12 @@ extern "C" int lb_adjoint_step(lb_ctx* c, long long nsteps, int checkpoint_every
           const int frc2 = fields_by_passes(a, Mn);
           if (frc2 != LB_OK) return frc2;
         } else {
-          a.adj_m = Mn;
+          adj_fields(a, Mn);
         }
         if (n < n1) {
           a.fout = rbp + (size_t)(1 - rc) * 2 * pbytes;
           a.gout = rbp + (size_t)(1 - rc) * 2 * pbytes + pbytes;
-          LB_CU(c, c->ops->fused(a, MODE_STEP, c->by, grid, st));
+          LB_CU(c, launch_step(c, a, MODE_STEP));
           rc ^= 1;
         }
       }

@@ -24,6 +24,13 @@ struct lb_ctx {
   double* fields = nullptr;  // [5][N] staging for host-bound lb_moments
   double* pops = nullptr;    // [38][N] staging for host-bound lb_populations
   double* pre = nullptr;     // FP64 form: [6][N] rho, 1/rho, j, psi of the state a step reads
+  // Form of the step. kTile: the tile march of lb_kernels.cuh, when the caller set its launch shape
+  // (tile_y or z_chunk); otherwise the three kernels of lb_split.cuh or the march of lb_march.cuh.
+  enum Form { kTile, kThree, kMarch } form = kTile;
+  void* fld = nullptr;       // kThree: its fields, [8] (FP64: [12]) [N] in the compute precision
+  int three_nt = 256;        // kThree: threads per CTA
+  int march_zc = 0;          // kMarch: planes per CTA
+  int nblk = 0;              // CTAs per plane: diagnostics partials per plane
   long long step = 0;
   // the current state is due for a Nu sample (nu_every) that the next step's launch takes in
   // passing (fused step + diagnostics); lb_nusselt, lb_diagnostics, lb_save and
@@ -51,6 +58,7 @@ inline int lb_cuda_fail(lb_ctx* c, const char* where, cudaError_t e) {
 // shared host helpers (lb_api.cu)
 tlbm::KArgs make_args(const lb_ctx* c);
 dim3 fused_grid(const lb_ctx* c);
+cudaError_t launch_step(const lb_ctx* c, const tlbm::KArgs& a, int mode);  // MODE_* over the whole cell
 int run_diag(lb_ctx* c, bool accumulate);
 int run_diag_acc(lb_ctx* c, double* acc);
 int finalize_diag(lb_ctx* c, double* acc);   // Nu(z) and health values from the partials

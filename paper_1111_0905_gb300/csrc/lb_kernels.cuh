@@ -9,7 +9,10 @@
 // Streaming: pull with two lattices (ping-pong). The buffer between steps holds the
 // post-collision populations f*(n); the state at time n+1 is their pull plus the wall rules.
 //
-// Fused step kernel: one CTA owns a 32 x BY column tile and a range of z planes and marches up
+// Forms of the step: the tile march below, for contexts whose caller set its launch shape; the three
+// kernels of lb_split.cuh and the march of lb_march.cuh for all others (choose_form in lb_api.cu).
+//
+// Tile march: one CTA owns a 32 x BY column tile and a range of z planes and marches up
 // in z. Per leading plane p it (M) pulls f on the tile plus a radius-2 ring and stores psi, rho,
 // j in shared memory; (U) for plane p-1 forms the force F and the physical velocity
 // u = (j + F/2)/rho on the tile plus a radius-1 ring; (C) for plane p-2 it pulls f and g of the
@@ -120,6 +123,12 @@ template <class R> struct KPar {
   R tau_nu, omega_nu, omega_kappa, G, g_z, lam, inv_cv, T_d, T_u, rho0, T0, E0;
   R va, vb, vT, vk;   // van der Waals-type psi: a, b, T_v, 2/(-G)
   R psi0, irho0;      // psi(rho0) = exp(-1/rho0) and 1/rho0 (deviation form of psi)
+  // three-kernel step: 1 - omega and, per class (rest, axis, diagonal), w omega, 3 w omega, 4.5 w omega
+  R om1, omk1, fo[3], fs[3], fq[3], go[3], gs[3], gq[3];
+  R mg, gz_u, gz_v;   // -G/12; g_z/2 and tau g_z
+  R src, lam45;       // 1/(2 c_v omega_kappa), 4.5 lam
+  R v_u, v_j;         // u' = v_u u + v_j j/rho: 2 tau and 1 - 2 tau
+  R ks;               // 1 - omega_nu/2 (Guo forcing)
 };
 
 // Scheme variants (comparisons with the paper's scheme, which is variant 0 of each).
@@ -154,6 +163,9 @@ struct KArgs {
   double* rho_out; double* ux_out; double* uy_out; double* uz_out; double* T_out;
   double* part;                       // [nz][ntiles][NPART] diagnostics partials (may be null)
   double* adj_m;                      // FP64 step: MF_* fields of the state read ([MF_COUNT][N]) or null
+  // three-kernel step (lb_split.cuh): fields in the compute precision, [N] each
+  void* fd_rho; void* fd_inv; void* fd_j[3]; void* fd_psi; void* fd_u[3]; void* fd_v[3];
+  unsigned div_m, div_s;              // i / nx = umulhi(i, div_m) >> div_s for i < 2^31 (0: nx = 1)
   double* pre;                        // FP64 form: rho, 1/rho, jx, jy, jz, psi of the state read ([6][N])
   KPar<double> pd;                    // the parameters above in double ...
   KPar<float> pf;                     // ... and in float

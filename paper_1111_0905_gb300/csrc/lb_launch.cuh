@@ -2,6 +2,7 @@
 // Each precision is compiled in its own translation unit (lb_prec_*.cu) that defines one table.
 #pragma once
 #include "lb_kernels.cuh"
+#include "lb_march.cuh"
 
 namespace tlbm {
 
@@ -18,6 +19,11 @@ struct PrecOps {
   cudaError_t (*info)(int by, int var, int out[4]);
   // store a given pre-collision state (float64 [19][N] f and g on the device) as the buffer
   cudaError_t (*setpops)(const KArgs&, const double*, const double*, cudaStream_t);
+  // the three-kernel step (lb_split.cuh) in mode MODE_* with CTAs of nt threads (64 or 256), and the
+  // one-launch march (lb_march.cuh) with chunks of zc planes and its tile height (0: none for FP64)
+  cudaError_t (*split)(const KArgs&, int mode, int nt, cudaStream_t);
+  cudaError_t (*march)(const KArgs&, int mode, int zc, cudaStream_t);
+  int march_ty;
   int slots;           // stored slots per lattice and node: 19, or 21 with the local references
 };
 
@@ -56,7 +62,8 @@ template <class S> struct OpsImpl {
     cudaError_t e;
     if ((e = attr_by<4>()) != cudaSuccess) return e;
     if ((e = attr_by<8>()) != cudaSuccess) return e;
-    return attr_by<16>();
+    if ((e = attr_by<16>()) != cudaSuccess) return e;
+    return march_prepare();
   }
   template <int BY, int VAR> static cudaError_t info_var(int out[4]) {
     if constexpr (!fits<BY>()) {
@@ -128,6 +135,105 @@ template <class S> struct OpsImpl {
     if (by == 8) return go_by<8>(a, mode, grid, st);
     if (by == 16) return go_by<16>(a, mode, grid, st);
     return cudaErrorInvalidValue;
+  }
+  // The three-kernel step (lb_split.cuh). NT threads per CTA: 256, or 64 for cells of few nodes per
+  // SM, which smaller CTAs spread more evenly (FP64 32^3: see the rule in lb_api.cu).
+  template <class... P, class... A> static cudaError_t follow(void (*k)(P...), unsigned grid, int nt, cudaStream_t st, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid); cfg.blockDim = dim3((unsigned)nt); cfg.stream = st;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at; cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k, args...);
+  }
+  template <int VAR, int NT> static cudaError_t three(const KArgs& a, int mode, cudaStream_t st) {
+    const int nb = (a.plane + NT - 1) / NT;
+    const unsigned grid = (unsigned)nb * (unsigned)a.nz;
+    cudaError_t e;
+    if ((e = follow(split_moments_kernel<S, (VAR & VAR_VDW) != 0, NT>, grid, NT, st, a, nb)) != cudaSuccess) return e;
+    if ((e = follow(split_velocity_kernel<R, VAR, NT>, grid, NT, st, a, nb)) != cudaSuccess) return e;
+    if (mode == MODE_STEP) return follow(split_collide_kernel<S, VAR, MODE_STEP, NT>, grid, NT, st, a, nb);
+    if (mode == MODE_MOMENTS) return follow(split_collide_kernel<S, VAR & VAR_VDW, MODE_MOMENTS, NT>, grid, NT, st, a, nb);
+    // the fused step + Nu sample exists for the paper's scheme only (the caller checks)
+    if constexpr (VAR == 0) return follow(split_collide_kernel<S, VAR, MODE_STEP_DIAG, NT>, grid, NT, st, a, nb);
+    else return cudaErrorInvalidValue;
+  }
+  template <int NT> static cudaError_t three_var(const KArgs& a, int mode, cudaStream_t st) {
+    switch (variant_of(a.forcing, a.psi_kind)) {
+      case 0: return three<0, NT>(a, mode, st);
+      case VAR_GUO: return three<VAR_GUO, NT>(a, mode, st);
+      case VAR_VDW: return three<VAR_VDW, NT>(a, mode, st);
+      default: return three<VAR_GUO | VAR_VDW, NT>(a, mode, st);
+    }
+  }
+  static cudaError_t split(const KArgs& a, int mode, int nt, cudaStream_t st) {
+    return nt == 64 ? three_var<64>(a, mode, st) : three_var<256>(a, mode, st);
+  }
+
+  // The one-launch step (lb_march.cuh). Tile heights: measured on the 256^3 and 512^3 boiling cells,
+  // FP32 7, 8, 9, 10, 12 rows: 0.99, 0.95, 1.03, 1.05, 1.13 ms and 8.0, 7.5, 7.3, 7.9, 8.5 ms; FP16
+  // deviations 7, 8, 9, 12 rows: 0.78, 0.72, 0.80, 0.95 ms at 256^3; local references 4, 5, 6, 7, 8
+  // rows: 1.27, 1.24, 1.86, 1.5, 1.80 ms (their 39 values in flight per thread spill beyond 5). Taller
+  // tiles recompute fewer ring nodes but leave fewer registers per thread.
+  static constexpr int MTY = IsLoc<S>::v ? 5 : 8;
+  template <int VAR, int MODE> static cudaError_t march_go(const KArgs& a, const MarchArgs& b, dim3 grid, cudaStream_t st) {
+    using GE = MarchGeo<S, MTY>;
+    split_march_kernel<S, VAR, MODE, MTY><<<grid, GE::NT, GE::smem, st>>>(a, b);
+    return cudaGetLastError();
+  }
+  template <int VAR, int MODE> static cudaError_t march_attr() {
+    return cudaFuncSetAttribute(split_march_kernel<S, VAR, MODE, MTY>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)MarchGeo<S, MTY>::smem);
+  }
+  static cudaError_t march_prepare() {
+    if constexpr (std::is_same<S, double>::value) {
+      return cudaSuccess;
+    } else {
+      cudaError_t e;
+      if ((e = march_attr<0, MODE_STEP>()) != cudaSuccess) return e;
+      if ((e = march_attr<VAR_GUO, MODE_STEP>()) != cudaSuccess) return e;
+      if ((e = march_attr<VAR_VDW, MODE_STEP>()) != cudaSuccess) return e;
+      if ((e = march_attr<VAR_GUO | VAR_VDW, MODE_STEP>()) != cudaSuccess) return e;
+      if ((e = march_attr<0, MODE_STEP_DIAG>()) != cudaSuccess) return e;
+      if ((e = march_attr<0, MODE_MOMENTS>()) != cudaSuccess) return e;
+      return march_attr<VAR_VDW, MODE_MOMENTS>();
+    }
+  }
+  static cudaError_t march(const KArgs& a, int mode, int zc, cudaStream_t st) {
+    if constexpr (std::is_same<S, double>::value) {
+      return cudaErrorInvalidValue;
+    } else {
+      MarchArgs b;
+      const long long es = (long long)sizeof(S), N = a.N, plane = a.plane;
+      for (int l = 0; l < Q + 2; ++l) {
+        b.fdst[l] = static_cast<char*>(a.fout) + l * N * es;
+        b.gdst[l] = static_cast<char*>(a.gout) + l * N * es;
+      }
+      for (int l = 0; l < Q; ++l) {
+        const long long src = (l * N - CZ(l) * plane) * es, ref = ((l == 0 ? Q : Q - 1 + CSQ(l)) * N - CZ(l) * plane) * es;
+        b.fsrc[l] = static_cast<const char*>(a.fin) + src;
+        b.gsrc[l] = static_cast<const char*>(a.gin) + src;
+        b.fref[l] = static_cast<const char*>(a.fin) + ref;
+        b.gref[l] = static_cast<const char*>(a.gin) + ref;
+      }
+      b.fref[Q] = static_cast<const char*>(a.fin) + (Q + 1) * N * es;
+      b.gref[Q] = static_cast<const char*>(a.gin) + (Q + 1) * N * es;
+      b.tiles_x = (a.nx + BX - 1) / BX;
+      b.zc = zc;
+      const dim3 grid((unsigned)(b.tiles_x * ((a.ny + MTY - 1) / MTY)), (unsigned)((a.nz + zc - 1) / zc));
+      const int var = variant_of(a.forcing, a.psi_kind);
+      if (mode == MODE_MOMENTS)
+        return (var & VAR_VDW) ? march_go<VAR_VDW, MODE_MOMENTS>(a, b, grid, st) : march_go<0, MODE_MOMENTS>(a, b, grid, st);
+      if (mode == MODE_STEP_DIAG)
+        return var == 0 ? march_go<0, MODE_STEP_DIAG>(a, b, grid, st) : cudaErrorInvalidValue;
+      switch (var) {
+        case 0: return march_go<0, MODE_STEP>(a, b, grid, st);
+        case VAR_GUO: return march_go<VAR_GUO, MODE_STEP>(a, b, grid, st);
+        case VAR_VDW: return march_go<VAR_VDW, MODE_STEP>(a, b, grid, st);
+        default: return march_go<VAR_GUO | VAR_VDW, MODE_STEP>(a, b, grid, st);
+      }
+    }
   }
   static int blocks_for(int N) {
     long long b = ((long long)N + 255) / 256;

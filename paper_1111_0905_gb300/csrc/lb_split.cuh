@@ -1,0 +1,404 @@
+// lb_split.cuh -- the time step as three streaming kernels, one node per thread:
+//
+//   moments   pull f; write rho (FP32 compute: drho; FP64: and 1/rho), j and psi;
+//   velocity  gather psi (Eq. (9)); write the physical velocity u = (j + F/2)/rho (FP64: and the
+//             equilibrium velocity u' = (j + tau F)/rho; Guo forcing: F in its place);
+//   collide   pull f and g, div(u) from six neighbours, collide and write both lattices.
+//
+// Nothing is recomputed and nothing waits at a barrier: the form of the FP64 step, which its FP64
+// instructions bound, and of the cells too small to fill the GPU with marching CTAs, where the
+// latency of one CTA's chain of planes is the time of the step.
+#pragma once
+#include "lb_kernels.cuh"
+
+namespace tlbm {
+
+// Node of a plane from its in-plane index: column x and row = y nx.
+struct NodePos {
+  unsigned x, row, i;
+  bool valid;
+};
+__device__ __forceinline__ NodePos node_at(const KArgs& a, unsigned i) {
+  NodePos n;
+  n.i = i;
+  n.valid = i < (unsigned)a.plane;
+  n.x = i - (a.div_m ? (__umulhi(i, a.div_m) >> a.div_s) : i) * (unsigned)a.nx;
+  n.row = i - n.x;
+  return n;
+}
+// columns x-1, x, x+1 and rows (y-1) nx, y nx, (y+1) nx of a node, periodic
+__device__ __forceinline__ void neighbours(unsigned (&xs)[3], unsigned (&ys)[3], const KArgs& a, unsigned x, unsigned row) {
+  const unsigned nx = (unsigned)a.nx, last = (unsigned)a.plane - nx;
+  xs[0] = x == 0 ? nx - 1 : x - 1; xs[1] = x; xs[2] = x + 1 == nx ? 0u : x + 1;
+  ys[0] = row == 0 ? last : row - nx; ys[1] = row; ys[2] = row == last ? 0u : row + nx;
+}
+
+// element i of a plane (the byte offset in a plane fits 32 bits)
+template <class T> __device__ __forceinline__ T ld_at(const T* base, unsigned i) {
+  return __ldg(reinterpret_cast<const T*>(reinterpret_cast<const char*>(base) + (size_t)(i * (unsigned)sizeof(T))));
+}
+template <> __device__ __forceinline__ half_loc ld_at<half_loc>(const half_loc* base, unsigned i) {
+  half_loc h;
+  h.h = __ldg(reinterpret_cast<const __half*>(reinterpret_cast<const char*>(base) + (size_t)(i * 2u)));
+  return h;
+}
+template <class T> __device__ __forceinline__ void st_at(T* base, unsigned i, T v) {
+  *reinterpret_cast<T*>(reinterpret_cast<char*>(base) + (size_t)(i * (unsigned)sizeof(T))) = v;
+}
+
+__device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+
+// 1/x: the division for FP64; for FP32 Newton's iteration on the hardware approximation (its error
+// is squared, so the result is within one rounding of 1/x for normal x, and the correctly rounded
+// intrinsic's test for its slow path is saved)
+__device__ __forceinline__ double recip(double x) { return 1.0 / x; }
+__device__ __forceinline__ float recip(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return fmaf(r, fmaf(-x, r, 1.0f), r);
+}
+
+// The 19 populations pulled at a node of plane z of lattice buf (through a wall the bounce-back
+// source), with the local references added.
+template <class S, class R>
+__device__ __forceinline__ void split_pull(R (&v)[Q], const S* __restrict__ buf, size_t N, size_t plane, int nz,
+                                           int z, const unsigned (&xs)[3], const unsigned (&ys)[3]) {
+  const unsigned own = xs[1] + ys[1];
+  S raw[Q];
+#pragma unroll
+  for (int l = 0; l < Q; ++l) {
+    const bool through = (CZ(l) > 0 && z == 0) || (CZ(l) < 0 && z == nz - 1);
+    const S* b = through ? buf + OPP(l) * N + (size_t)z * plane : buf + l * N + (size_t)(z - CZ(l)) * plane;
+    raw[l] = ld_at(b, through ? own : xs[1 - CX(l)] + ys[1 - CY(l)]);
+  }
+#pragma unroll
+  for (int l = 0; l < Q; ++l) v[l] = cvt<S, R>(raw[l]);
+  if constexpr (IsLoc<S>::v) {
+    const S* r1 = buf + (size_t)Q * N;
+    const S* r2 = buf + (size_t)(Q + 1) * N;
+    const size_t zo = (size_t)z * plane;
+    v[0] += 12.0f * (cvt<S, R>(ld_at(r1 + zo, own)) - cvt<S, R>(ld_at(r2 + zo, own)));
+#pragma unroll
+    for (int l = 1; l < Q; ++l) {
+      const bool through = (CZ(l) > 0 && z == 0) || (CZ(l) < 0 && z == nz - 1);
+      const size_t zs = through ? zo : (size_t)(z - CZ(l)) * plane;
+      v[l] += cvt<S, R>(ld_at((CSQ(l) == 1 ? r1 : r2) + zs, through ? own : xs[1 - CX(l)] + ys[1 - CY(l)]));
+    }
+  }
+}
+
+// Density and momentum deviations from the sums and differences of the opposite pairs (39 additions
+// instead of 45 term by term; the differences of like numbers come first).
+template <class R>
+__device__ __forceinline__ void pair_moments(const R (&f)[Q], R& drho, R& jx, R& jy, R& jz) {
+  R s[Q / 2], d[Q / 2];
+#pragma unroll
+  for (int k = 0; k < Q / 2; ++k) { s[k] = f[2 * k + 1] + f[2 * k + 2]; d[k] = f[2 * k + 1] - f[2 * k + 2]; }
+  drho = ((f[0] + (s[0] + s[1])) + (s[2] + s[3])) + ((s[4] + s[5]) + (s[6] + (s[7] + s[8])));
+  jx = d[0] + ((d[3] + d[4]) + (d[5] + d[6]));
+  jy = d[1] + ((d[3] - d[4]) + (d[7] + d[8]));
+  jz = d[2] + ((d[5] - d[6]) + (d[7] - d[8]));
+}
+// 12 sum_l W_l c_l psi(x + c_l) from the nine pair differences d_k = psi(x + c_l) - psi(x - c_l),
+// l = 2k + 1: twice the axis pair's plus the diagonal pairs' (W = 1/6, 1/12)
+template <class R>
+__device__ __forceinline__ void pair_gradient(const R (&d)[Q / 2], R& ax, R& ay, R& az) {
+  ax = R(2) * d[0] + ((d[3] + d[4]) + (d[5] + d[6]));
+  ay = R(2) * d[1] + ((d[3] - d[4]) + (d[7] + d[8]));
+  az = R(2) * d[2] + ((d[5] - d[6]) + (d[7] - d[8]));
+}
+
+// psi of a node as the fields keep it (FP32 compute, the paper's psi: its deviation from psi(rho0))
+template <class R, bool VDW>
+__device__ __forceinline__ R split_psi(R rho, R drho, R inv, const KPar<R>& kp) {
+  if constexpr (VDW) return psi_vdw(rho, kp);
+  else if constexpr (sizeof(R) == 8) return fexp(-inv);
+  else return kp.psi0 * expm1_dev(drho * inv * kp.irho0);
+}
+// -G psi / 12 from psi as kept
+template <class R, bool VDW>
+__device__ __forceinline__ R split_mg(R psi, const KPar<R>& kp) {
+  return kp.mg * ((sizeof(R) == 4 && !VDW) ? kp.psi0 + psi : psi);
+}
+
+// BGK relaxation of one lattice towards its equilibrium around the velocity v, pair by pair:
+//   out_l = om1 in_l + [ev + 9 (c.v)(c.F')] +- [s (c.v) + 3 (c.F')],  ev = q (c.v)^2 + P per class,
+// F' = 0 without Guo forcing. in(l) and put(l, value) access the populations.
+template <class R, bool GUO, class In, class Put>
+__device__ __forceinline__ void relax(R om1, const R (&P)[3], const R (&q)[3], const R (&s)[3], R vx, R vy, R vz,
+                                      const R (&F)[3], R ks, In in, Put put) {
+  put(0, fma_rn(om1, in(0), P[0]));
+#pragma unroll
+  for (int l = 1; l < Q; l += 2) {
+    const R cv = cdot<R>(l, vx, vy, vz);
+    R ev = fma_rn(q[CLS(l)] * cv, cv, P[CLS(l)]);
+    if constexpr (GUO) {
+      const R cF = (WT<R>(l) * ks) * cdot<R>(l, F[0], F[1], F[2]);
+      ev = ev + R(9) * cv * cF;
+      const R od = fma_rn(s[CLS(l)], cv, R(3) * cF);
+      put(l, fma_rn(om1, in(l), ev) + od);
+      put(OPP(l), fma_rn(om1, in(OPP(l)), ev) - od);
+    } else {
+      put(l, fma_rn(s[CLS(l)], cv, fma_rn(om1, in(l), ev)));
+      put(OPP(l), fma_rn(-s[CLS(l)], cv, fma_rn(om1, in(OPP(l)), ev)));
+    }
+  }
+}
+// g towards g^eq(rho, T, u) with the counter term; D2 = 2 div(u). Per class (rest, axis, diagonal)
+// P = go [dE - 1.5 E u.u - E div(u)/(c_v omk) + (|c|^2 - 1) tg], tg = 4.5 (lam (T - T0) - dE/3).
+template <class R, class In, class Put>
+__device__ __forceinline__ void relax_g(const KPar<R>& kp, R E, R dE, R drho, R inv, R D2, R ux, R uy, R uz, In in, Put put) {
+  const R uu = ux * ux + uy * uy + uz * uz;
+  const R b0 = dE - E * (R(1.5) * uu + D2 * kp.src);
+  const R tg = kp.lam45 * ((dE - kp.T0 * drho) * inv) - R(1.5) * dE;
+  const R P[3] = {kp.go[0] * (b0 - tg), kp.go[1] * b0, kp.go[2] * (b0 + tg)};
+  const R q[3] = {R(0), kp.gq[1] * E, kp.gq[2] * E}, s[3] = {R(0), kp.gs[1] * E, kp.gs[2] * E};
+  const R F[3] = {R(0), R(0), R(0)};
+  relax<R, false>(kp.omk1, P, q, s, ux, uy, uz, F, R(0), in, put);
+}
+// f towards f^eq(rho, u', T) (w = u'), or with Guo forcing towards f^eq(rho, u, T) plus its source
+// (w = F). a0 = drho - 1.5 rho v.v, th = 4.5 (rho (T - 1/3) - rho0 (T0 - 1/3)) = 4.5 (dE - drho/3).
+template <class R, bool GUO, class In, class Put>
+__device__ __forceinline__ void relax_f(const KPar<R>& kp, R rho, R drho, R dE, R ux, R uy, R uz, const R (&w)[3], In in, Put put) {
+  const R vx = GUO ? ux : w[0], vy = GUO ? uy : w[1], vz = GUO ? uz : w[2];
+  const R vv = vx * vx + vy * vy + vz * vz;
+  const R a0 = drho - (R(1.5) * rho) * vv;
+  const R th = R(4.5) * dE - R(1.5) * drho;
+  R P[3] = {kp.fo[0] * (a0 - th), kp.fo[1] * a0, kp.fo[2] * (a0 + th)};
+  const R q[3] = {R(0), kp.fq[1] * rho, kp.fq[2] * rho}, s[3] = {R(0), kp.fs[1] * rho, kp.fs[2] * rho};
+  if constexpr (GUO) {
+    // (1 - om/2) w_l [3 (c - u).F + 9 (c.u)(c.F)]: the part -3 u.F of the even terms
+    const R uF = R(-3) * kp.ks * (ux * w[0] + uy * w[1] + uz * w[2]);
+    P[0] += WT<R>(0) * uF; P[1] += WT<R>(1) * uF; P[2] += WT<R>(7) * uF;
+  }
+  relax<R, GUO>(kp.om1, P, q, s, vx, vy, vz, w, kp.ks, in, put);
+}
+
+// One node's terms of the diagnostics: rho U u_z, T, rho, rho T, minima and the non-finite flag.
+// U = c_v T + int_0^rho P_NI/s^2 ds: (G/4) e^{-2/rho}, or -T_v ln(1 - b rho) - a rho (vdW).
+template <class R> struct DiagTerms {
+  R conv = R(0), T = R(0), rho = R(0), E = R(0), mr = R(sizeof(R) == 8 ? 1e300 : 3.0e38), mT = mr;
+  bool bad = false;
+  template <bool VDW>
+  __device__ __forceinline__ void take(const KArgs& a, R r, R inv, R t, R e, R ux, R uy, R uz) {
+    const KPar<R>& kp = kpar<R>(a);
+    R U;
+    if constexpr (sizeof(R) == 8)
+      U = a.c_v * t + (VDW ? -kp.vT * log(1.0 - kp.vb * r) - kp.va * r : 0.25 * a.G * exp(-2.0 / r));
+    else
+      U = R(a.c_v) * t + (VDW ? -kp.vT * logf(R(1) - kp.vb * r) - kp.va * r : R(0.25) * kp.G * fexp(R(-2) * inv));
+    conv = r * U * uz;
+    T = t; rho = r; E = e; mr = r; mT = t;
+    bad = !(isfinite(r) && isfinite(t) && isfinite(ux) && isfinite(uy) && isfinite(uz));
+  }
+  // warp sums in the compute precision into red[7][NW] (column w)
+  template <int NW> __device__ __forceinline__ void reduce(R (&red)[7][NW], int w, int lane) {
+    conv = warp_sum(conv); T = warp_sum(T); rho = warp_sum(rho); E = warp_sum(E);
+    mr = warp_min(mr); mT = warp_min(mT);
+    const int nbad = __popc(__ballot_sync(0xffffffffu, bad));
+    if (lane == 0) {
+      red[0][w] = conv; red[1][w] = T; red[2][w] = rho; red[3][w] = E; red[4][w] = mr; red[5][w] = mT;
+      red[6][w] = R(nbad);
+    }
+  }
+};
+// partial q of one CTA's plane piece, over its warps in order, in FP64
+template <class R, int NW>
+__device__ __forceinline__ void diag_combine(const R (&red)[7][NW], int q, double* part) {
+  double acc = double(red[q][0]);
+  for (int k = 1; k < NW; ++k) acc = (q == 4 || q == 5) ? fmin(acc, double(red[q][k])) : acc + double(red[q][k]);
+  part[q] = acc;
+}
+
+// The kernels of one step follow each other closely: each is launched as its predecessor's CTAs end
+// (programmatic dependent launch) and waits here, before its first access to memory, until all of the
+// predecessor's results are there. (FP32 32^3: 14.7 us a step without, 7.6 us with. Letting the
+// successor up earlier, while the predecessor still runs, only crowds its CTAs: FP64 32^3 28 -> 54 us.)
+__device__ __forceinline__ void wait_for_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// ---- kernels: nb CTAs of NT threads per plane ---------------------------------------------------
+template <class S, bool VDW, int NT>
+__global__ void __launch_bounds__(NT) split_moments_kernel(const KArgs a, int nb) {
+  using R = typename Store<S>::R;
+  constexpr bool F64 = sizeof(R) == 8;
+  const int z = (int)blockIdx.x / nb;
+  const NodePos n = node_at(a, (blockIdx.x - (unsigned)(z * nb)) * NT + threadIdx.x);
+  wait_for_predecessor();
+  if (!n.valid) return;
+  unsigned xs[3], ys[3];
+  neighbours(xs, ys, a, n.x, n.row);
+  R f[Q];
+  split_pull<S, R>(f, static_cast<const S*>(a.fin), (size_t)a.N, (size_t)a.plane, a.nz, z, xs, ys);
+  R drho, jx, jy, jz;
+  pair_moments<R>(f, drho, jx, jy, jz);
+  const KPar<R>& kp = kpar<R>(a);
+  const R rho = kp.rho0 + drho;
+  const R inv = recip(rho);
+  const size_t zo = (size_t)z * (size_t)a.plane;
+  st_at(static_cast<R*>(a.fd_rho) + zo, n.i, F64 ? rho : drho);
+  if constexpr (F64) st_at(static_cast<R*>(a.fd_inv) + zo, n.i, inv);
+  st_at(static_cast<R*>(a.fd_j[0]) + zo, n.i, jx);
+  st_at(static_cast<R*>(a.fd_j[1]) + zo, n.i, jy);
+  st_at(static_cast<R*>(a.fd_j[2]) + zo, n.i, jz);
+  st_at(static_cast<R*>(a.fd_psi) + zo, n.i, split_psi<R, VDW>(rho, drho, inv, kp));
+}
+
+template <class R, int VAR, int NT>
+__global__ void __launch_bounds__(NT) split_velocity_kernel(const KArgs a, int nb) {
+  constexpr bool GUO = (VAR & VAR_GUO) != 0, VDW = (VAR & VAR_VDW) != 0, F64 = sizeof(R) == 8;
+  const int z = (int)blockIdx.x / nb;
+  const NodePos n = node_at(a, (blockIdx.x - (unsigned)(z * nb)) * NT + threadIdx.x);
+  wait_for_predecessor();
+  if (!n.valid) return;
+  unsigned xs[3], ys[3];
+  neighbours(xs, ys, a, n.x, n.row);
+  const size_t zo = (size_t)z * (size_t)a.plane;
+  // radius 1: the mirror image of a plane beyond a wall is the wall plane itself
+  const R* p0 = static_cast<const R*>(a.fd_psi) + zo;
+  const R* pm = z > 0 ? p0 - a.plane : p0;
+  const R* pp = z + 1 < a.nz ? p0 + a.plane : p0;
+  R d[Q / 2];
+#pragma unroll
+  for (int k = 0; k < Q / 2; ++k) {
+    const int l = 2 * k + 1;
+    const R* hi = CZ(l) == 0 ? p0 : (CZ(l) > 0 ? pp : pm);
+    const R* lo = CZ(l) == 0 ? p0 : (CZ(l) > 0 ? pm : pp);
+    d[k] = ld_at(hi, xs[1 + CX(l)] + ys[1 + CY(l)]) - ld_at(lo, xs[1 - CX(l)] + ys[1 - CY(l)]);
+  }
+  R A[3];
+  pair_gradient<R>(d, A[0], A[1], A[2]);
+  const KPar<R>& kp = kpar<R>(a);
+  const R rv = ld_at(static_cast<const R*>(a.fd_rho) + zo, n.i);
+  const R rho = F64 ? rv : kp.rho0 + rv;
+  R inv;
+  if constexpr (F64) inv = ld_at(static_cast<const R*>(a.fd_inv) + zo, n.i);
+  else inv = recip(rho);
+  const R mg = split_mg<R, VDW>(ld_at(p0, n.i), kp);              // F = mg A + rho g_z z
+  const R mi = mg * inv;
+  const R mu = R(0.5) * mi, mv = kp.tau_nu * mi;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const R j = ld_at(static_cast<const R*>(a.fd_j[k]) + zo, n.i);
+    const R ji = j * inv;
+    st_at(static_cast<R*>(a.fd_u[k]) + zo, n.i, mu * A[k] + (k == 2 ? ji + kp.gz_u : ji));
+    if constexpr (F64) {
+      if constexpr (GUO) st_at(static_cast<R*>(a.fd_v[k]) + zo, n.i, k == 2 ? mg * A[k] + rho * kp.g_z : mg * A[k]);
+      else st_at(static_cast<R*>(a.fd_v[k]) + zo, n.i, mv * A[k] + (k == 2 ? ji + kp.gz_v : ji));
+    }
+  }
+  if constexpr (F64) {
+    if (a.adj_m != nullptr) {
+#pragma unroll
+      for (int k = 0; k < 3; ++k) st_at(a.adj_m + (MF_AX + k) * (size_t)a.N + zo, n.i, A[k] * (1.0 / 12.0));
+    }
+  }
+}
+
+// Resident 256-thread CTAs per SM that the collision's registers allow. FP32: 64 registers (4 CTAs;
+// 256^3 boiling cell 0.84 ms against 0.90 with 3 and 0.97 with 2); 16-bit 80 (3); FP64 128 (2).
+template <class S> constexpr int split_mb() { return sizeof(S) == 4 ? 4 : (sizeof(S) == 2 ? 3 : 2); }
+
+// MODE_MOMENTS: the fields of the state read instead of the collision; DIAG modes: the partials of
+// the state read, one set per CTA.
+template <class S, int VAR, int MODE, int NT>
+__global__ void __launch_bounds__(NT, split_mb<S>() * 256 / NT) split_collide_kernel(const KArgs a, int nb) {
+  using R = typename Store<S>::R;
+  constexpr bool GUO = (VAR & VAR_GUO) != 0, VDW = (VAR & VAR_VDW) != 0, F64 = sizeof(R) == 8;
+  constexpr bool COLLIDE = MODE != MODE_MOMENTS, DIAG = MODE != MODE_STEP;
+  constexpr int NW = NT / 32;
+  const int z = (int)blockIdx.x / nb;
+  const NodePos n = node_at(a, (blockIdx.x - (unsigned)(z * nb)) * NT + threadIdx.x);
+  wait_for_predecessor();
+  const size_t N = (size_t)a.N, plane = (size_t)a.plane, zo = (size_t)z * plane;
+  const KPar<R>& kp = kpar<R>(a);
+  const unsigned o = n.i;
+  DiagTerms<R> dt;
+  if (n.valid) {
+    const S* fin = static_cast<const S*>(a.fin);
+    const S* gin = static_cast<const S*>(a.gin);
+    R g[Q], f[Q];
+    unsigned xs[3], ys[3];
+    neighbours(xs, ys, a, n.x, n.row);
+    split_pull<S, R>(g, gin, N, plane, a.nz, z, xs, ys);
+    if constexpr (COLLIDE) split_pull<S, R>(f, fin, N, plane, a.nz, z, xs, ys);
+    const R* pux = static_cast<const R*>(a.fd_u[0]) + zo;
+    const R* puy = static_cast<const R*>(a.fd_u[1]) + zo;
+    const R* puz = static_cast<const R*>(a.fd_u[2]) + zo;
+    const R rv = ld_at(static_cast<const R*>(a.fd_rho) + zo, o);
+    const R ux = ld_at(pux, o), uy = ld_at(puy, o), uz = ld_at(puz, o);
+    R inv;
+    if constexpr (F64) inv = ld_at(static_cast<const R*>(a.fd_inv) + zo, o);
+    if (z == 0 || z == a.nz - 1)
+      g_wall_fix<S, R>(g, fin, a.N, (int)(zo + o), z, a.nz, kp.rho0, kp.T0, kp.T_d, kp.T_u, kp.lam);
+    const R rho = F64 ? rv : kp.rho0 + rv;
+    const R drho = F64 ? rv - kp.rho0 : rv;
+    if constexpr (!F64) inv = recip(rho);
+    R dE = g[0];
+#pragma unroll
+    for (int l = 1; l < Q; ++l) dE = dE + g[l];
+    const R E = kp.E0 + dE;
+    const R T = E * inv;            // the plain step needs it for the adjoint's fields only
+    if constexpr (DIAG) dt.template take<VDW>(a, rho, inv, T, E, ux, uy, uz);
+    if constexpr (COLLIDE) {
+      const R uzp = z + 1 < a.nz ? ld_at(puz + plane, o) : -uz;
+      const R uzm = z > 0 ? ld_at(puz - plane, o) : -uz;
+      // 2 div(u)
+      const R D2 = ((ld_at(pux, xs[2] + ys[1]) - ld_at(pux, xs[0] + ys[1])) +
+                    (ld_at(puy, xs[1] + ys[2]) - ld_at(puy, xs[1] + ys[0]))) + (uzp - uzm);
+      // u' (Guo forcing: F). FP32 compute: from u = (j + F/2)/rho and j of the pulled f, which saves
+      // writing and reading three fields; FP64 reads them (its FP64 instructions cost more)
+      R w[3];
+      if constexpr (F64) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) w[k] = ld_at(static_cast<const R*>(a.fd_v[k]) + zo, o);
+      } else {
+        R dr, j[3];
+        pair_moments<R>(f, dr, j[0], j[1], j[2]);
+        const R u[3] = {ux, uy, uz};
+        const R c = inv * kp.v_j;           // (1 - 2 tau)/rho
+#pragma unroll
+        for (int k = 0; k < 3; ++k) w[k] = GUO ? R(2) * (rho * u[k] - j[k]) : kp.v_u * u[k] + c * j[k];
+      }
+      S* __restrict__ fo = static_cast<S*>(a.fout) + zo;
+      S* __restrict__ go = static_cast<S*>(a.gout) + zo;
+      R lrf[3] = {R(0), R(0), R(0)}, lrg[3] = {R(0), R(0), R(0)};
+      auto put = [&](S* base, int l, R v) {
+        Store<S>::st(reinterpret_cast<S*>(reinterpret_cast<char*>(base + l * N) + (size_t)(o * (unsigned)sizeof(S))), v);
+      };
+      if constexpr (IsLoc<S>::v) {
+        float a1, a2, b1, b2;
+        loc_refs_of<S>(drho, dE, T - kp.T0, kp.lam, a1, a2, b1, b2);
+        lrf[0] = 12.0f * (a1 - a2); lrf[1] = a1; lrf[2] = a2;
+        lrg[0] = 12.0f * (b1 - b2); lrg[1] = b1; lrg[2] = b2;
+        put(fo, Q, a1); put(fo, Q + 1, a2); put(go, Q, b1); put(go, Q + 1, b2);
+      }
+      if constexpr (F64) {
+        if (a.adj_m != nullptr) {
+          st_at(a.adj_m + MF_T * N + zo, o, T);
+          st_at(a.adj_m + MF_D * N + zo, o, 0.5 * D2);
+        }
+      }
+      relax_g<R>(kp, E, dE, drho, inv, D2, ux, uy, uz, [&](int l) { return g[l]; },
+                 [&](int l, R v) { put(go, l, IsLoc<S>::v ? v - lrg[CSQ(l)] : v); });
+      relax_f<R, GUO>(kp, rho, drho, dE, ux, uy, uz, w, [&](int l) { return f[l]; },
+                      [&](int l, R v) { put(fo, l, IsLoc<S>::v ? v - lrf[CSQ(l)] : v); });
+    } else {
+      if (a.rho_out) st_at(a.rho_out + zo, o, double(rho));
+      if (a.ux_out) st_at(a.ux_out + zo, o, double(ux));
+      if (a.uy_out) st_at(a.uy_out + zo, o, double(uy));
+      if (a.uz_out) st_at(a.uz_out + zo, o, double(uz));
+      if (a.T_out) st_at(a.T_out + zo, o, double(T));
+    }
+  }
+  if constexpr (DIAG) {
+    if (a.part != nullptr) {
+      __shared__ R red[7][NW];
+      dt.template reduce<NW>(red, threadIdx.x >> 5, threadIdx.x & 31);
+      __syncthreads();
+      if (threadIdx.x < 7) diag_combine<R, NW>(red, (int)threadIdx.x, a.part + (size_t)blockIdx.x * NPART);
+    }
+  }
+}
+
+}  // namespace tlbm
