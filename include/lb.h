@@ -156,7 +156,7 @@ int lb_nusselt(lb_ctx* ctx, double* nu_mean, double* nu_z, double* nu_time_avg);
  * sweep). J is accumulated in the reverse sweep from the identity Nu_mean = 1 + sum_x rho U u_z /
  * (kappa (T_d - T_u) nx ny) (the conduction term telescopes). Output pointers may be NULL.
  * Device memory: nsteps/checkpoint_every + 1 population checkpoints, checkpoint_every + 1 sets of
- * 20 float64 fields, 3 float64 states and 15 float64 fields, allocated and freed by the call.
+ * 20 float64 fields, 3 float64 states and 17 float64 fields, allocated and freed by the call.
  * checkpoint_every = 0 takes the longest segment whose buffers fit in 85 % of the device's free
  * memory: all nsteps states' fields when they fit (with FP64 storage nothing is then recomputed),
  * else the largest length that fits.

@@ -9,7 +9,9 @@
 //   streaming^T (push of lambda_{n+1}, bounce-back transposed, the thermal wall rule's density
 //   and T_w terms) -> collision^T (f^eq(rho, u', T), g^eq(rho, T, u), counter term) -> the Nu
 //   terms of state n -> divergence^T (radius-1 gather) -> velocities^T (u, u' -> j, F, rho) ->
-//   force^T (radius-1 psi gather with the mirrored wall ghosts; dJ/dG) -> moments^T.
+//   force^T (radius-1 psi gather with the mirrored wall ghosts; dJ/dG) -> moments^T
+// in three kernels: coll_adj (up to the Nu terms), vel_adj (divergence^T, velocities^T and the own
+// node's part of force^T), force_adj (the gather and the new lambda).
 // The forward states are recomputed per segment from checkpoints taken every K steps; the
 // macroscopic fields of a state are recomputed per reverse step.
 #include <cuda_runtime.h>
@@ -24,23 +26,48 @@
 namespace tlbm {
 namespace adj {
 
-struct Geom { int nx, ny, nz, plane, N; };
+struct Geom {
+  int nx, ny, nz, plane, N, nb;   // nb = CTAs per plane
+  unsigned div_m, div_s;          // as KArgs::div_m, div_s
+};
 struct Par {
   double tau, om, omk, G, gz, lam, cv, kappa, Td, Tu;
+  double om1, omk1;            // 1 - om, 1 - omk
+  double w[3], j3[2], q9[2];   // f: om w per class; 3 om w and 9 om w of the axis and diagonal classes
+  double wg[3], j3g[2], q9g[2];  // the same of g
   double Kc;        // 1 / (N_t kappa (T_d - T_u) nx ny): weight of sum_x rho U u_z in J
+  double src;       // -1 / (omk c_v)
   int include_nu;   // add (1/N_t) dNu_mean/dx of this state
 };
 
 // fields of M (forward macros of one state, MF_* of lb_kernels.cuh), each [N]
-// fields of A (adjoints of the macros), each [N]
-enum { AF_RHO = 0, AF_T, AF_UX, AF_UY, AF_UZ, AF_VX, AF_VY, AF_VZ, AF_D, AF_FX, AF_FY, AF_FZ, AF_JX, AF_JY,
-       AF_JZ, AF_COUNT };
-// per-block parameter partials
+// fields of A (adjoints of the macros), each [N]: of coll_adj (first block), of vel_adj (second; RHO
+// is updated): dJ/dE, dJ/dj, H = psi dJ/dF and the factor of the gathered sum in dJ/drho
+enum { AF_RHO = 0, AF_T, AF_UX, AF_UY, AF_UZ, AF_VX, AF_VY, AF_VZ, AF_D,
+       AF_E, AF_JX, AF_JY, AF_JZ, AF_HX, AF_HY, AF_HZ, AF_KP, AF_COUNT };
+// per-block parameter partials: wall terms of dJ/dT_d and dJ/dT_u, dJ/dG, the sum of J
 enum { P_TD = 0, P_TU, P_G, P_J, P_COUNT };
 
-constexpr int kBlocks = 1024;
 constexpr int kThreads = 256;
 
+// node of this thread: one CTA covers kThreads consecutive nodes of a plane
+struct Node {
+  unsigned xs[3], ys[3];   // columns x-1, x, x+1 and rows (y-1) nx, y nx, (y+1) nx, periodic
+  unsigned i;              // in-plane index
+  int z;
+  bool valid;
+};
+__device__ __forceinline__ Node node_of(const Geom& g) {
+  Node n;
+  n.z = (int)blockIdx.x / g.nb;
+  n.i = (blockIdx.x - (unsigned)(n.z * g.nb)) * kThreads + threadIdx.x;
+  n.valid = n.i < (unsigned)g.plane;
+  const unsigned nx = (unsigned)g.nx, last = (unsigned)g.plane - nx;
+  const unsigned x = n.i - (g.div_m ? (__umulhi(n.i, g.div_m) >> g.div_s) : n.i) * nx, row = n.i - x;
+  n.xs[0] = x == 0 ? nx - 1 : x - 1; n.xs[1] = x; n.xs[2] = x + 1 == nx ? 0u : x + 1;
+  n.ys[0] = row == 0 ? last : row - nx; n.ys[1] = row; n.ys[2] = row == last ? 0u : row + nx;
+  return n;
+}
 __device__ __forceinline__ void coords(int idx, const Geom& g, int& x, int& y, int& z) {
   x = idx % g.nx;
   y = (idx / g.nx) % g.ny;
@@ -50,15 +77,18 @@ __device__ __forceinline__ int at(const Geom& g, int x, int y, int z) {
   return z * g.plane + wrapi(y, g.ny) * g.nx + wrapi(x, g.nx);
 }
 
-__device__ double block_sum(double v, double* sh) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  __syncthreads();
-  if (lane == 0) sh[w] = v;
+// Sum of v over the CTA on thread 0, in a fixed order: every warp leaves its values in shared memory
+// and one adds them, 8 per lane and then by shuffles (12 FP64 instructions of one warp instead of 5
+// of every warp). sh is the caller's own array.
+__device__ __forceinline__ double block_sum(double v, double* sh) {
+  sh[threadIdx.x] = v;
   __syncthreads();
   double s = 0.0;
-  if (threadIdx.x == 0)
-    for (int k = 0; k < (int)(blockDim.x >> 5); ++k) s += sh[k];
+  if (threadIdx.x < 32) {
+    s = sh[threadIdx.x];
+    for (int k = 32; k < kThreads; k += 32) s += sh[threadIdx.x + k];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  }
   return s;
 }
 
@@ -121,229 +151,223 @@ __global__ void div_fwd_kernel(Geom g, double* __restrict__ M) {
   }
 }
 
-// streaming^T, wall rules^T, collision^T and the Nu terms, per node
-// adjoint of post-collision population l at node (x, y, z): lambda'_l(x + c_l), or through a wall
-// the bounce-back that delivered f*_l(x) as f'_{opp(l)}(x) (g: with a minus sign)
-__device__ __forceinline__ void adj_pull(const double* __restrict__ Ln, const Geom& g, int l, int i,
-                                         int x, int y, int z, double& lf, double& lg) {
-  const size_t N = g.N;
-  const int zn = z + CZ(l);
-  if (zn < 0 || zn >= g.nz) {
-    lf = Ln[OPP(l) * N + i];
-    lg = -Ln[(Q + OPP(l)) * N + i];
-  } else {
-    const int j = at(g, x + CX(l), y + CY(l), zn);
-    lf = Ln[l * N + j];
-    lg = Ln[(Q + l) * N + j];
+// streaming^T: adjoint of the post-collision populations l = 0..18 at node n in lattice Ln (f or g):
+// lambda'_l(x + c_l), or through a wall the bounce-back that delivered f*_l(x) as f'_{opp(l)}(x) (g:
+// with a minus sign)
+template <bool G_LATTICE>
+__device__ __forceinline__ void adj_pull(double (&v)[Q], const double* __restrict__ Ln, const Geom& g, const Node& n) {
+  const size_t N = (size_t)g.N, plane = (size_t)g.plane;
+#pragma unroll
+  for (int l = 0; l < Q; ++l) {
+    const int zn = n.z + CZ(l);
+    const bool wall = zn < 0 || zn >= g.nz;
+    const double* b = wall ? Ln + OPP(l) * N + (size_t)n.z * plane : Ln + l * N + (size_t)zn * plane;
+    const double x = __ldg(b + (wall ? n.i : n.xs[1 + CX(l)] + n.ys[1 + CY(l)]));
+    v[l] = G_LATTICE && wall ? -x : x;
   }
 }
 
-// collision^T, one node per thread. The populations are taken in pairs (l, opp(l)), whose
-// equilibria share the part even in c_l and differ in sign in the odd part: with s = a_l + a_opp
-// and d = a_l - a_opp the pair contributes s (even part) + d (odd part) to each adjoint.
-__global__ void __launch_bounds__(256) coll_adj_kernel(const double* __restrict__ X, const double* __restrict__ M,
-                                                       const double* __restrict__ Ln, Geom g, Par p,
-                                                       double* __restrict__ L, double* __restrict__ A,
-                                                       double* __restrict__ part) {
-  __shared__ double sh[32];
-  const size_t N = g.N;
+// Moments in c_l of the adjoint populations, weighted as the equilibria's terms are: sums per class
+// (rest, axis, diagonal), 3 sum w om c_l a_l and 9 sum w om c_l c_l a_l. Every term of collision^T is
+// polynomial in c_l of degree <= 2, so these ten numbers per lattice carry all of it.
+struct AdjMoments {
+  double s0, s1, s2;                 // om w sum of a over the class
+  double jx, jy, jz;
+  double qxx, qyy, qzz, qxy, qxz, qyz;
+};
+__device__ __forceinline__ AdjMoments adj_moments(const double (&a)[Q], const double (&w)[3], const double (&j3)[2],
+                                                  const double (&q9)[2]) {
+  double S[Q / 2], D[Q / 2];
+#pragma unroll
+  for (int k = 0; k < Q / 2; ++k) { S[k] = a[2 * k + 1] + a[2 * k + 2]; D[k] = a[2 * k + 1] - a[2 * k + 2]; }
+  // pairs: 0..2 axis x, y, z; 3, 4 xy (same, opposite signs); 5, 6 xz; 7, 8 yz
+  const double Pxy = S[3] + S[4], Pxz = S[5] + S[6], Pyz = S[7] + S[8];
+  AdjMoments m;
+  m.s0 = w[0] * a[0];
+  m.s1 = w[1] * ((S[0] + S[1]) + S[2]);
+  m.s2 = w[2] * ((Pxy + Pxz) + Pyz);
+  m.jx = j3[0] * D[0] + j3[1] * ((D[3] + D[4]) + (D[5] + D[6]));
+  m.jy = j3[0] * D[1] + j3[1] * ((D[3] - D[4]) + (D[7] + D[8]));
+  m.jz = j3[0] * D[2] + j3[1] * ((D[5] - D[6]) + (D[7] - D[8]));
+  m.qxx = q9[0] * S[0] + q9[1] * (Pxy + Pxz);
+  m.qyy = q9[0] * S[1] + q9[1] * (Pxy + Pyz);
+  m.qzz = q9[0] * S[2] + q9[1] * (Pxz + Pyz);
+  m.qxy = q9[1] * (S[3] - S[4]);
+  m.qxz = q9[1] * (S[5] - S[6]);
+  m.qyz = q9[1] * (S[7] - S[8]);
+  return m;
+}
+
+// Wall rules^T, collision^T and the Nu terms. Bound by its FP64 instructions like everything here; the
+// moment form takes about 200 of them a node where the sum over the pairs took 650 (64^3: 128 us against
+// 288; the three reverse kernels 226 us against 388).
+__global__ void __launch_bounds__(kThreads) coll_adj_kernel(const double* __restrict__ M, const double* __restrict__ Ln,
+                                                            Geom g, Par p, double* __restrict__ A,
+                                                            double* __restrict__ part) {
+  __shared__ double sh[4][kThreads];
+  const Node n = node_of(g);
+  const size_t N = (size_t)g.N, i = (size_t)n.z * (size_t)g.plane + n.i;
+  const bool wallz = n.z == 0 || n.z == g.nz - 1;
   double pTd = 0.0, pTu = 0.0, pG = 0.0, pJ = 0.0;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < g.N; i += gridDim.x * blockDim.x) {
-    int x, y, z;
-    coords(i, g, x, y, z);
+  if (n.valid) {
     const double rho = M[MF_RHO * N + i], T = M[MF_T * N + i], E = rho * T;
     const double ux = M[MF_UX * N + i], uy = M[MF_UY * N + i], uz = M[MF_UZ * N + i];
-    const double vx = M[MF_VX * N + i], vy = M[MF_VY * N + i], vz = M[MF_VZ * N + i];
-    const double D = M[MF_D * N + i];
-    double a_rho = 0.0;
+    double a_rho = 0.0, a_T = 0.0, a_D = 0.0;
+    double a_v[3] = {0.0, 0.0, 0.0}, a_u[3] = {0.0, 0.0, 0.0};
     if (Ln) {
-      // thermal wall rule: g'_m(x_w) = ... + 2 w_m [rho T_w + 4.5 (lam T_w - rho T_w/3)(|c_m|^2-1)]
+      double a[Q];
+      adj_pull<false>(a, Ln, g, n);
+      // f* = (1 - om) f + om f^eq(rho, v, T), f^eq = w rho [1 + 3 c.v + 4.5 (c.v)^2 - 1.5 v.v + 4.5 (T - 1/3) k]
+      {
+        const AdjMoments m = adj_moments(a, p.w, p.j3, p.q9);
+        const double vx = M[MF_VX * N + i], vy = M[MF_VY * N + i], vz = M[MF_VZ * N + i];
+        const double vv = vx * vx + vy * vy + vz * vz;
+        const double sf = (m.s0 + m.s1) + m.s2, sfk = m.s2 - m.s0;
+        const double qx = m.qxx * vx + m.qxy * vy + m.qxz * vz, qy = m.qxy * vx + m.qyy * vy + m.qyz * vz,
+                     qz = m.qxz * vx + m.qyz * vy + m.qzz * vz;
+        a_rho = sf * (1.0 - 1.5 * vv) + sfk * (4.5 * T - 1.5);
+        a_rho += vx * (0.5 * qx + m.jx) + vy * (0.5 * qy + m.jy) + vz * (0.5 * qz + m.jz);
+        a_T = 4.5 * rho * sfk;
+        const double s3 = 3.0 * sf;
+        a_v[0] = rho * (m.jx + qx - s3 * vx); a_v[1] = rho * (m.jy + qy - s3 * vy); a_v[2] = rho * (m.jz + qz - s3 * vz);
+      }
+      // g* = (1 - omk) g + omk g^eq(rho, T, u) + w S, S = -rho T D / c_v,
+      // g^eq = w [rho T (1 + 3 c.u + 4.5 (c.u)^2 - 1.5 u.u) + 4.5 (lam T - rho T/3) k]
+      adj_pull<true>(a, Ln + Q * N, g, n);
+      {
+        const AdjMoments m = adj_moments(a, p.wg, p.j3g, p.q9g);
+        const double uu = ux * ux + uy * uy + uz * uz;
+        const double sg = (m.s0 + m.s1) + m.s2, sgk = m.s2 - m.s0;
+        const double qx = m.qxx * ux + m.qxy * uy + m.qxz * uz, qy = m.qxy * ux + m.qyy * uy + m.qyz * uz,
+                     qz = m.qxz * ux + m.qyz * uy + m.qzz * uz;
+        const double X = sg * (1.0 - 1.5 * uu) +
+                         (ux * (0.5 * qx + m.jx) + uy * (0.5 * qy + m.jy) + uz * (0.5 * qz + m.jz));
+        const double lS = p.src * sg;          // sum_l w_l lambda_l = sg/omk, times -1/c_v
+        const double D = M[MF_D * N + i];
+        a_rho += T * (X - 1.5 * sgk + lS * D);
+        a_T += rho * (X + lS * D) + (4.5 * p.lam - 1.5 * rho) * sgk;
+        a_D = lS * E;
+        const double s3 = 3.0 * sg;
+        a_u[0] = E * (m.jx + qx - s3 * ux); a_u[1] = E * (m.jy + qy - s3 * uy); a_u[2] = E * (m.jz + qz - s3 * uz);
+      }
+      if (wallz) {
+        // thermal wall rule: g'_m(x_w) = ... + 2 w_m [rho T_w + 4.5 (lam T_w - rho T_w/3)(|c_m|^2-1)]
 #pragma unroll
-      for (int m = 0; m < Q; ++m) {
-        const bool bot = (CZ(m) > 0 && z == 0), top = (CZ(m) < 0 && z == g.nz - 1);
-        if (bot || top) {
-          const double Tw = bot ? p.Td : p.Tu;
-          const double lm = Ln[(Q + m) * N + i];
-          const double k = CSQ(m) - 1;
-          a_rho += 2.0 * WT<double>(m) * Tw * (1.0 - 1.5 * k) * lm;
-          const double dTw = 2.0 * WT<double>(m) * (rho + 4.5 * (p.lam - rho / 3.0) * k) * lm;
-          if (bot) pTd += dTw; else pTu += dTw;
+        for (int m = 0; m < Q; ++m) {
+          const bool bot = (CZ(m) > 0 && n.z == 0), top = (CZ(m) < 0 && n.z == g.nz - 1);
+          if (bot || top) {
+            const double Tw = bot ? p.Td : p.Tu;
+            const double lm = Ln[(Q + m) * N + i];
+            const double k = CSQ(m) - 1;
+            a_rho += 2.0 * WT<double>(m) * Tw * (1.0 - 1.5 * k) * lm;
+            const double dTw = 2.0 * WT<double>(m) * (rho + 4.5 * (p.lam - rho / 3.0) * k) * lm;
+            if (bot) pTd += dTw; else pTu += dTw;
+          }
         }
       }
     }
-    // collision^T: f* = (1 - om) f + om f^eq(rho, v, T), g* = (1 - omk) g + omk g^eq(rho, T, u) + w S
-    const double vv = vx * vx + vy * vy + vz * vz, uu = ux * ux + uy * uy + uz * uz;
-    double a_T = 0.0, lS = 0.0;
-    double sfk = 0.0, sf = 0.0, sg = 0.0;          // sums of s_f k, s_f and s_g over the pairs
-    double avx = 0.0, avy = 0.0, avz = 0.0, aux = 0.0, auy = 0.0, auz = 0.0;
-    const double Tm = 4.5 * (T - 1.0 / 3.0), lk = 4.5 * (p.lam - rho / 3.0);
-    const double ev0 = 1.0 - 1.5 * vv, eu0 = 1.0 - 1.5 * uu;   // the velocity-squared parts
-#pragma unroll
-    for (int l = 0; l < Q; ++l) {
-      if (l != 0 && (l & 1) == 0) continue;    // with its odd partner
-      const int o = (l == 0) ? 0 : OPP(l);
-      double lf = 0.0, lg = 0.0, lfo = 0.0, lgo = 0.0;
-      if (Ln) {
-        adj_pull(Ln, g, l, i, x, y, z, lf, lg);
-        if (l != 0) adj_pull(Ln, g, o, i, x, y, z, lfo, lgo);
-      }
-      L[l * N + i] = (1.0 - p.om) * lf;
-      L[(Q + l) * N + i] = (1.0 - p.omk) * lg;
-      if (l != 0) {
-        L[o * N + i] = (1.0 - p.om) * lfo;
-        L[(Q + o) * N + i] = (1.0 - p.omk) * lgo;
-      }
-      // class factor k = |c_l|^2 - 1 (-1 rest, 0 axis, +1 diagonal) taken by branches that fold,
-      // so that no multiply by k is executed
-      const int kc = CSQ(l) - 1;
-      const double w = WT<double>(l);
-      const double af = p.om * w * lf, ag = p.omk * w * lg;
-      // f^eq: even 1 + 4.5 (c.v)^2 - 1.5 v.v + 4.5 (T - 1/3) k, odd 3 c.v; d/dT 4.5 k rho;
-      // d/dv rho (3 c + 9 (c.v) c - 3 v)
-      // g^eq: rho T P(u) + 4.5 (lam T - rho T/3) k, P even 1 + 4.5 (c.u)^2 - 1.5 u.u, odd 3 c.u
-      if (l == 0) {
-        // the rest population (c = 0, k = -1): even parts only
-        a_rho += af * (ev0 - Tm) + T * (ag * (eu0 + 1.5));
-        a_T += rho * (ag * eu0) - ag * lk;
-        sfk -= af;
-        sf += af;
-        sg += ag;
-        lS += w * lg;
-      } else {
-        const double cv = cdot<double>(l, vx, vy, vz);
-        const double cu = cdot<double>(l, ux, uy, uz);
-        const double afo = p.om * w * lfo, ago = p.omk * w * lgo;
-        const double s_f = af + afo, d_f = af - afo, s_g = ag + ago, d_g = ag - ago;
-        const double evf = kc == 0 ? ev0 : ev0 + Tm;          // axis: k = 0, diagonal: k = 1
-        a_rho += s_f * (evf + 4.5 * cv * cv) + d_f * (3.0 * cv);
-        if (kc != 0) sfk += s_f;
-        sf += s_f;
-        const double ef = 3.0 * d_f + 9.0 * s_f * cv;
-        cadd<double>(l, ef, avx, avy, avz);
-        const double Pe = eu0 + 4.5 * cu * cu, Po = 3.0 * cu;
-        const double Pk = kc == 0 ? Pe : Pe - 1.5;
-        a_rho += T * (s_g * Pk + d_g * Po);
-        a_T += rho * (s_g * Pe + d_g * Po);
-        if (kc != 0) a_T += s_g * lk;
-        sg += s_g;
-        const double eg = 3.0 * d_g + 9.0 * s_g * cu;
-        cadd<double>(l, eg, aux, auy, auz);
-        lS += w * (lg + lgo);
-      }
-    }
-    a_T += 4.5 * rho * sfk;
-    double a_v[3] = {rho * (avx - 3.0 * vx * sf), rho * (avy - 3.0 * vy * sf), rho * (avz - 3.0 * vz * sf)};
-    double a_u[3] = {E * (aux - 3.0 * ux * sg), E * (auy - 3.0 * uy * sg), E * (auz - 3.0 * uz * sg)};
-    // counter term S = -rho T D / c_v
-    a_rho += lS * (-T * D / p.cv);
-    a_T += lS * (-rho * D / p.cv);
-    const double a_D = lS * (-E / p.cv);
     // Nu terms: J_n = (1/N_t)[1 + sum_x rho U u_z / (kappa (T_d - T_u) nx ny)], U = c_v T + (G/4) e^{-2/rho}
     if (p.include_nu) {
       const double psi = M[MF_PSI * N + i];
       const double e2 = psi * psi;            // e^{-2/rho} = psi^2
       const double U = p.cv * T + 0.25 * p.G * e2;
-      a_rho += p.Kc * (U * uz + uz * 0.5 * p.G * e2 / rho);
-      a_T += p.Kc * rho * p.cv * uz;
-      a_u[2] += p.Kc * rho * U;
-      pG += p.Kc * rho * uz * 0.25 * e2;
-      pJ += p.Kc * rho * U * uz;       // J = 1 + sum_n sum_x Kc rho U u_z (conduction telescopes)
-      const double conv = p.Kc * rho * U * uz / (p.Td - p.Tu);
-      pTd -= conv;
-      pTu += conv;
+      const double ku = p.Kc * uz, kr = p.Kc * rho;
+      a_rho += ku * U;        // and the derivative of e^{-2/rho}, which vel_adj adds (it has 1/rho)
+      a_T += kr * p.cv * uz;
+      a_u[2] += kr * U;
+      pG = kr * uz * 0.25 * e2;
+      pJ = kr * U * uz;       // J = 1 + sum_n sum_x Kc rho U u_z (conduction telescopes)
     }
     A[AF_RHO * N + i] = a_rho; A[AF_T * N + i] = a_T; A[AF_D * N + i] = a_D;
-    A[AF_UX * N + i] = a_u[0]; A[AF_UY * N + i] = a_u[1]; A[AF_UZ * N + i] = a_u[2];
-    A[AF_VX * N + i] = a_v[0]; A[AF_VY * N + i] = a_v[1]; A[AF_VZ * N + i] = a_v[2];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) { A[(AF_UX + k) * N + i] = a_u[k]; A[(AF_VX + k) * N + i] = a_v[k]; }
   }
-  const double s0 = block_sum(pTd, sh), s1 = block_sum(pTu, sh), s2 = block_sum(pG, sh);
-  const double s3 = block_sum(pJ, sh);
-  if (threadIdx.x == 0) {
-    part[blockIdx.x * P_COUNT + P_TD] += s0;
-    part[blockIdx.x * P_COUNT + P_TU] += s1;
-    part[blockIdx.x * P_COUNT + P_G] += s2;
-    part[blockIdx.x * P_COUNT + P_J] += s3;
+  double* o = part + (size_t)blockIdx.x * P_COUNT;
+  if (p.include_nu) {
+    const double s2 = block_sum(pG, sh[0]), s3 = block_sum(pJ, sh[1]);
+    if (threadIdx.x == 0) { o[P_G] += s2; o[P_J] += s3; }
+  }
+  if (wallz && Ln) {
+    const double s0 = block_sum(pTd, sh[2]), s1 = block_sum(pTu, sh[3]);
+    if (threadIdx.x == 0) { o[P_TD] += s0; o[P_TU] += s1; }
   }
 }
 
-// divergence^T (radius-1 gather) and velocities^T: u = (j + F/2)/rho, u' = (j + tau F)/rho
-__global__ void vel_adj_kernel(const double* __restrict__ M, Geom g, Par p, double* __restrict__ A) {
-  const size_t N = g.N;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < g.N; i += gridDim.x * blockDim.x) {
-    int x, y, z;
-    coords(i, g, x, y, z);
-    double lu[3] = {A[AF_UX * N + i], A[AF_UY * N + i], A[AF_UZ * N + i]};
-    lu[0] += 0.5 * (A[AF_D * N + at(g, x - 1, y, z)] - A[AF_D * N + at(g, x + 1, y, z)]);
-    lu[1] += 0.5 * (A[AF_D * N + at(g, x, y - 1, z)] - A[AF_D * N + at(g, x, y + 1, z)]);
-    const double dm = (z >= 1) ? A[AF_D * N + i - g.plane] : A[AF_D * N + i];
-    const double dp = (z <= g.nz - 2) ? A[AF_D * N + i + g.plane] : A[AF_D * N + i];
-    lu[2] += 0.5 * (dm - dp);
-    const double inv = 1.0 / M[MF_RHO * N + i];   // one division per node on the FP64 pipe
-    double a_rho = A[AF_RHO * N + i];
-    for (int a = 0; a < 3; ++a) {
-      const double lv = A[(AF_VX + a) * N + i];
-      A[(AF_JX + a) * N + i] = (lv + lu[a]) * inv;
-      A[(AF_FX + a) * N + i] = (p.tau * lv + 0.5 * lu[a]) * inv;
-      a_rho -= (M[(MF_VX + a) * N + i] * lv + M[(MF_UX + a) * N + i] * lu[a]) * inv;
+// divergence^T (radius-1 gather), velocities^T: u = (j + F/2)/rho, u' = (j + tau F)/rho, the node's own
+// factors of force^T: F = -G psi A + rho g_z z, psi = e^{-1/rho}, and T = E/rho ^T
+__global__ void __launch_bounds__(kThreads) vel_adj_kernel(const double* __restrict__ M, Geom g, Par p,
+                                                           double* __restrict__ A, double* __restrict__ part) {
+  __shared__ double sh[kThreads];
+  const Node n = node_of(g);
+  const size_t N = (size_t)g.N, plane = (size_t)g.plane, zo = (size_t)n.z * plane, i = zo + n.i;
+  double pG = 0.0;
+  if (n.valid) {
+    const double* aD = A + AF_D * N;
+    const double own = aD[i];
+    const double dm = n.z >= 1 ? aD[i - plane] : own, dp = n.z <= g.nz - 2 ? aD[i + plane] : own;
+    const double gr[3] = {aD[zo + n.xs[0] + n.ys[1]] - aD[zo + n.xs[2] + n.ys[1]],
+                          aD[zo + n.xs[1] + n.ys[0]] - aD[zo + n.xs[1] + n.ys[2]], dm - dp};
+    const double rho = M[MF_RHO * N + i], psi = M[MF_PSI * N + i];
+    const double inv = 1.0 / rho;
+    double dot = 0.0, FA = 0.0, lFz = 0.0;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const double lu = A[(AF_UX + k) * N + i] + 0.5 * gr[k], lv = A[(AF_VX + k) * N + i];
+      A[(AF_JX + k) * N + i] = (lv + lu) * inv;
+      const double lF = (p.tau * lv + 0.5 * lu) * inv;
+      dot += M[(MF_VX + k) * N + i] * lv + M[(MF_UX + k) * N + i] * lu;
+      FA += lF * M[(MF_AX + k) * N + i];
+      A[(AF_HX + k) * N + i] = psi * lF;
+      if (k == 2) lFz = lF;
     }
+    const double aE = A[AF_T * N + i] * inv;
+    const double kp = -p.G * psi * inv * inv;       // lambda_psi -> lambda_rho of the terms -G (...)
+    pG = -psi * FA;
+    A[AF_E * N + i] = aE;
+    A[AF_KP * N + i] = kp * (1.0 / 12.0);
+    double a_rho = A[AF_RHO * N + i] - dot * inv + p.gz * lFz + kp * FA - aE * M[MF_T * N + i];
+    if (p.include_nu) a_rho += p.Kc * M[MF_UZ * N + i] * (0.5 * p.G * psi * psi) * inv;
     A[AF_RHO * N + i] = a_rho;
   }
-}
-
-// c_l . (lambda_Fx, lambda_Fy, lambda_Fz) at node j, loading only the components c_l has
-__device__ __forceinline__ double cdot_at(int l, const double* __restrict__ A, size_t N, int j) {
-  const double x = CX(l) != 0 ? A[AF_FX * N + j] : 0.0;
-  const double y = CY(l) != 0 ? A[AF_FY * N + j] : 0.0;
-  const double z = CZ(l) != 0 ? A[AF_FZ * N + j] : 0.0;
-  return cdot<double>(l, x, y, z);
-}
-
-// force^T (psi gather with mirrored ghosts), psi^T, T = E/rho ^T and moments^T
-__global__ void force_adj_kernel(const double* __restrict__ M, Geom g, Par p,
-                                 const double* __restrict__ A, double* __restrict__ L,
-                                 double* __restrict__ part) {
-  __shared__ double sh[32];
-  const size_t N = g.N;
-  double pG = 0.0;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < g.N; i += gridDim.x * blockDim.x) {
-    int x, y, z;
-    coords(i, g, x, y, z);
-    const double psi = M[MF_PSI * N + i], rho = M[MF_RHO * N + i], T = M[MF_T * N + i];
-    const double lF[3] = {A[AF_FX * N + i], A[AF_FY * N + i], A[AF_FZ * N + i]};
-    // own psi factor of F(x) = -G psi(x) A(x)
-    double lpsi = -p.G * (lF[0] * M[MF_AX * N + i] + lF[1] * M[MF_AY * N + i] + lF[2] * M[MF_AZ * N + i]);
-    pG -= psi * (lF[0] * M[MF_AX * N + i] + lF[1] * M[MF_AY * N + i] + lF[2] * M[MF_AZ * N + i]);
-    // psi(y) enters F(x) for every (x, l) with mirror(x + c_l) = y
-#pragma unroll
-    for (int l = 1; l < Q; ++l) {
-      const double W = FW<double>(l);
-      const int zi = z - CZ(l);          // interior link x = y - c_l
-      if (zi >= 0 && zi < g.nz) {
-        const int j = at(g, x - CX(l), y - CY(l), zi);
-        const double cl = cdot_at(l, A, N, j);
-        lpsi += -p.G * W * cl * M[MF_PSI * N + j];
-      }
-      const int zg = z + CZ(l);          // ghost link: x in this plane, x + c_l beyond a wall
-      if (CZ(l) != 0 && (zg < 0 || zg >= g.nz)) {
-        const int j = at(g, x - CX(l), y - CY(l), z);
-        const double cl = cdot_at(l, A, N, j);
-        lpsi += -p.G * W * cl * M[MF_PSI * N + j];
-      }
-    }
-    const double inv = 1.0 / rho;
-    double a_rho = A[AF_RHO * N + i] + p.gz * lF[2] + lpsi * psi * inv * inv;
-    const double a_T = A[AF_T * N + i];
-    const double a_E = a_T * inv;
-    a_rho -= a_T * T * inv;
-    const double lj[3] = {A[AF_JX * N + i], A[AF_JY * N + i], A[AF_JZ * N + i]};
-#pragma unroll
-    for (int l = 0; l < Q; ++l) {
-      L[l * N + i] += (l == 0) ? a_rho : a_rho + cdot<double>(l, lj[0], lj[1], lj[2]);
-      L[(Q + l) * N + i] += a_E;
-    }
-  }
   const double s = block_sum(pG, sh);
-  if (threadIdx.x == 0) part[blockIdx.x * P_COUNT + P_G] += s;
+  if (threadIdx.x == 0) part[(size_t)blockIdx.x * P_COUNT + P_G] += s;
+}
+
+// force^T's gather and moments^T. psi(y) enters F(x) for every link x + c_l = y: sum_l W_l c_l . H(y - c_l);
+// a ghost link of a wall plane (x + c_l beyond the wall, its mirror image y) is the same sum over the
+// plane's mirror image with H_z negated. Then lambda_l = (1 - om) lambda*_l + a_rho + c_l . a_j (g: + a_E).
+__global__ void __launch_bounds__(kThreads) force_adj_kernel(const double* __restrict__ A, const double* __restrict__ Ln,
+                                                             Geom g, Par p, double* __restrict__ L) {
+  const Node n = node_of(g);
+  if (!n.valid) return;
+  const size_t N = (size_t)g.N, plane = (size_t)g.plane, zo = (size_t)n.z * plane, i = zo + n.i;
+  const double *Hx = A + AF_HX * N + zo, *Hy = A + AF_HY * N + zo, *Hz = A + AF_HZ * N + zo;
+  auto at2 = [&](const double* f, int dx, int dy) { return f[n.xs[1 + dx] + n.ys[1 + dy]]; };
+  double s = 2.0 * ((at2(Hx, -1, 0) - at2(Hx, 1, 0)) + (at2(Hy, 0, -1) - at2(Hy, 0, 1)));
+  s += ((at2(Hx, -1, -1) + at2(Hy, -1, -1)) - (at2(Hx, 1, 1) + at2(Hy, 1, 1))) +
+       ((at2(Hx, -1, 1) - at2(Hy, -1, 1)) - (at2(Hx, 1, -1) - at2(Hy, 1, -1)));
+#pragma unroll
+  for (int dz = -1; dz <= 1; dz += 2) {
+    const bool wall = n.z + dz < 0 || n.z + dz >= g.nz;
+    const long long off = wall ? 0 : dz * (long long)plane;
+    const double *hx = Hx + off, *hy = Hy + off, *hz = Hz + off;
+    s += (at2(hx, -1, 0) - at2(hx, 1, 0)) + (at2(hy, 0, -1) - at2(hy, 0, 1));
+    const double t = 2.0 * at2(hz, 0, 0) + ((at2(hz, -1, 0) + at2(hz, 1, 0)) + (at2(hz, 0, -1) + at2(hz, 0, 1)));
+    s = ((dz < 0) != wall) ? s + t : s - t;
+  }
+  const double a_rho = A[AF_RHO * N + i] + A[AF_KP * N + i] * s;
+  const double jx = A[AF_JX * N + i], jy = A[AF_JY * N + i], jz = A[AF_JZ * N + i];
+  double a[Q];
+  if (Ln) adj_pull<false>(a, Ln, g, n);
+#pragma unroll
+  for (int l = 0; l < Q; ++l) {
+    const double c = l == 0 ? a_rho : a_rho + cdot<double>(l, jx, jy, jz);
+    L[l * N + i] = Ln ? p.om1 * a[l] + c : c;
+  }
+  const double aE = A[AF_E * N + i];
+  if (Ln) adj_pull<true>(a, Ln + Q * N, g, n);
+#pragma unroll
+  for (int l = 0; l < Q; ++l) L[(Q + l) * N + i] = Ln ? p.omk1 * a[l] + aE : aE;
 }
 
 // dJ/dT0 from lambda_0: x_0 = (f^eq(rho0, 0, T0), g^eq(rho0, T0, 0))
@@ -400,12 +424,14 @@ extern "C" int lb_adjoint_step(lb_ctx* c, long long nsteps, int checkpoint_every
   const size_t pbytes = (size_t)c->ops->slots * N * c->ops->esize;
   const size_t sbytes = 2 * (size_t)Q * N * sizeof(double);
   const size_t mstate = (size_t)MF_COUNT * N;   // doubles per state's fields
+  const int nbp = (c->plane + kThreads - 1) / kThreads;
+  const size_t parts = (size_t)nbp * (size_t)c->p.nz;      // CTAs of a reverse kernel
   // device bytes of the call for segment length k (the allocations below)
   auto bytes_for = [&](long long k) -> double {
     const double nck_k = (double)((nsteps + k - 1) / k);
     return nck_k * 2.0 * (double)pbytes + 4.0 * (double)pbytes + 64.0 + 3.0 * (double)sbytes +
            (double)(k + 1) * (double)mstate * 8.0 + (double)AF_COUNT * (double)N * 8.0 +
-           (double)kBlocks * P_COUNT * 8.0 + (dJ_dT0 ? (double)N * 8.0 : 0.0);
+           (double)parts * P_COUNT * 8.0 + (dJ_dT0 ? (double)N * 8.0 : 0.0);
   };
   long long K = checkpoint_every < nsteps ? checkpoint_every : nsteps;
   if (checkpoint_every == 0) {
@@ -422,7 +448,8 @@ extern "C" int lb_adjoint_step(lb_ctx* c, long long nsteps, int checkpoint_every
   }
   const long long nck = (nsteps + K - 1) / K;
   cudaStream_t st = c->stream;
-  Geom g{c->p.nx, c->p.ny, c->p.nz, c->plane, c->N};
+  const KArgs a0 = make_args(c);
+  Geom g{c->p.nx, c->p.ny, c->p.nz, c->plane, c->N, nbp, a0.div_m, a0.div_s};
 
   // FP64 storage: the step writes the fields of the state it reads (adj_m), so the reverse sweep
   // needs no separate moments, force and divergence passes; other storage recomputes them in
@@ -435,7 +462,7 @@ extern "C" int lb_adjoint_step(lb_ctx* c, long long nsteps, int checkpoint_every
       cudaMalloc(&mb.p, (size_t)(K + 1) * mstate * sizeof(double)) != cudaSuccess ||
       cudaMalloc(&ab.p, (size_t)AF_COUNT * N * sizeof(double)) != cudaSuccess ||
       cudaMalloc(&lb.p, 2 * sbytes) != cudaSuccess ||
-      cudaMalloc(&pt.p, (size_t)kBlocks * P_COUNT * sizeof(double)) != cudaSuccess ||
+      cudaMalloc(&pt.p, parts * P_COUNT * sizeof(double)) != cudaSuccess ||
       (dJ_dT0 && cudaMalloc(&d0.p, N * sizeof(double)) != cudaSuccess))
     return lb_fail(c, LB_ENOMEM, "adjoint buffers");
   unsigned char* ckp = static_cast<unsigned char*>(ck.p);
@@ -445,15 +472,25 @@ extern "C" int lb_adjoint_step(lb_ctx* c, long long nsteps, int checkpoint_every
   double* A = static_cast<double*>(ab.p);
   double* Lb[2] = {static_cast<double*>(lb.p), static_cast<double*>(lb.p) + 2 * Q * N};
   double* part = static_cast<double*>(pt.p);
-  LB_CU(c, cudaMemsetAsync(part, 0, (size_t)kBlocks * P_COUNT * sizeof(double), st));
+  LB_CU(c, cudaMemsetAsync(part, 0, parts * P_COUNT * sizeof(double), st));
   const int frc = flush_sample(c);    // a Nu sample due for the time average of lb_nusselt
   if (frc) return frc;
 
   const double dT = c->p.T_d - c->p.T_u;
-  Par par{c->p.tau_nu, 1.0 / c->p.tau_nu, 1.0 / c->p.tau_kappa, c->p.G, c->p.g_z, c->lam, c->p.c_v,
-          c->p.kappa, c->p.T_d, c->p.T_u,
-          1.0 / ((double)nsteps * c->p.kappa * dT * (double)c->p.nx * (double)c->p.ny), 0};
-  const int nb = (int)std::min<long long>(kBlocks, ((long long)N + kThreads - 1) / kThreads);
+  Par par;
+  std::memset(&par, 0, sizeof(par));
+  par.tau = c->p.tau_nu; par.om = 1.0 / c->p.tau_nu; par.omk = 1.0 / c->p.tau_kappa; par.G = c->p.G; par.gz = c->p.g_z;
+  par.lam = c->lam; par.cv = c->p.c_v; par.kappa = c->p.kappa; par.Td = c->p.T_d; par.Tu = c->p.T_u;
+  par.om1 = 1.0 - par.om; par.omk1 = 1.0 - par.omk;
+  const double wc[3] = {1.0 / 3.0, 1.0 / 18.0, 1.0 / 36.0};
+  for (int k = 0; k < 3; ++k) { par.w[k] = par.om * wc[k]; par.wg[k] = par.omk * wc[k]; }
+  for (int k = 0; k < 2; ++k) {
+    par.j3[k] = 3.0 * par.w[k + 1]; par.q9[k] = 9.0 * par.w[k + 1];
+    par.j3g[k] = 3.0 * par.wg[k + 1]; par.q9g[k] = 9.0 * par.wg[k + 1];
+  }
+  par.src = -1.0 / (par.omk * par.cv);
+  par.Kc = 1.0 / ((double)nsteps * c->p.kappa * dT * (double)c->p.nx * (double)c->p.ny);
+  const int nb = (int)std::min<long long>(1024, ((long long)N + kThreads - 1) / kThreads);   // grid-stride passes
   // fields of a state from its storage image (a.fin, a.gin) by the separate FP64 passes
   auto fields_by_passes = [&](const KArgs& a, double* Mn) -> int {
     LB_CU(c, c->ops->pops(a, X, X + Q * N, st));
@@ -517,9 +554,10 @@ extern "C" int lb_adjoint_step(lb_ctx* c, long long nsteps, int checkpoint_every
       const double* Mn = Ms + (size_t)(n - n0) * mstate;
       par.include_nu = (n >= 1) ? 1 : 0;
       double* Lcur = Lb[1 - li];
-      coll_adj_kernel<<<nb, kThreads, 0, st>>>(nullptr, Mn, have_next ? Lb[li] : nullptr, g, par, Lcur, A, part);
-      vel_adj_kernel<<<nb, kThreads, 0, st>>>(Mn, g, par, A);
-      force_adj_kernel<<<nb, kThreads, 0, st>>>(Mn, g, par, A, Lcur, part);
+      const double* Lnext = have_next ? Lb[li] : nullptr;
+      coll_adj_kernel<<<(unsigned)parts, kThreads, 0, st>>>(Mn, Lnext, g, par, A, part);
+      vel_adj_kernel<<<(unsigned)parts, kThreads, 0, st>>>(Mn, g, par, A, part);
+      force_adj_kernel<<<(unsigned)parts, kThreads, 0, st>>>(A, Lnext, g, par, Lcur);
       LB_CU(c, cudaGetLastError());
       li = 1 - li;
       have_next = true;
@@ -529,16 +567,18 @@ extern "C" int lb_adjoint_step(lb_ctx* c, long long nsteps, int checkpoint_every
       LB_CU(c, cudaGetLastError());
     }
   }
-  std::vector<double> hp((size_t)kBlocks * P_COUNT);
+  std::vector<double> hp(parts * P_COUNT);
   LB_CU(c, cudaMemcpyAsync(hp.data(), part, hp.size() * sizeof(double), cudaMemcpyDeviceToHost, st));
   if (dJ_dT0) LB_CU(c, cudaMemcpyAsync(dJ_dT0, d0.p, N * sizeof(double), cudaMemcpyDeviceToHost, st));
   LB_CU(c, cudaStreamSynchronize(st));
   double s[P_COUNT] = {0.0, 0.0, 0.0, 0.0};
-  for (int b = 0; b < kBlocks; ++b)
-    for (int k = 0; k < P_COUNT; ++k) s[k] += hp[(size_t)b * P_COUNT + k];
+  for (size_t b = 0; b < parts; ++b)
+    for (int k = 0; k < P_COUNT; ++k) s[k] += hp[b * P_COUNT + k];
+  // the convective terms sum_x rho U u_z / (T_d - T_u) of Nu depend on the wall temperatures as well
+  const double conv = s[P_J] / (par.Td - par.Tu);
   if (J) *J = 1.0 + s[P_J];
-  if (dJ_dTd) *dJ_dTd = s[P_TD];
-  if (dJ_dTu) *dJ_dTu = s[P_TU];
+  if (dJ_dTd) *dJ_dTd = s[P_TD] - conv;
+  if (dJ_dTu) *dJ_dTu = s[P_TU] + conv;
   if (dJ_dG) *dJ_dG = s[P_G];
   return LB_OK;
 }
