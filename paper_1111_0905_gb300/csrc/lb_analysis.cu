@@ -6,6 +6,7 @@
 // integers.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <vector>
 
@@ -26,36 +27,55 @@ __device__ double block_sum(double v, double* sh) {
   return s;
 }
 
-// One block per plane z: sums of rho, T and P div(u), P = rho T + (G/2) e^{-2/rho} (or, for
-// the van der Waals psi, rho T + rho^2 (b T_v/(1 - b rho) - a)), div(u) by central differences
-// with u_z -> -u_z across the walls (the step's divergence).
-__global__ void profiles_kernel(const double* __restrict__ rho, const double* __restrict__ ux,
+// Four sums over the CTA, one warp adding each from shared memory in a fixed order; sum k is returned to
+// warp k.
+constexpr int kThreads = 256, kWarps = kThreads / 32;
+__device__ __forceinline__ double block_sum4(const double (&v)[4], double (&sh)[4][kThreads]) {
+#pragma unroll
+  for (int k = 0; k < 4; ++k) sh[k][threadIdx.x] = v[k];
+  __syncthreads();
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  double s = 0.0;
+  if (w < 4) {
+    s = sh[w][lane];
+    for (int k = 32; k < kThreads; k += 32) s += sh[w][lane + k];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  }
+  return s;
+}
+
+// CTA z np + p: sums over part p of plane z of rho, T and P div(u), P = rho T + (G/2) e^{-2/rho} (or,
+// for the van der Waals psi, rho T + rho^2 (b T_v/(1 - b rho) - a)), div(u) by central differences
+// with u_z -> -u_z across the walls (the step's divergence). Bound by FP64 instructions (exp, the
+// division); with one CTA per plane 96 planes left a third of the SMs idle (108 -> 77 us at 96^3).
+__global__ void profiles_kernel(int np, const double* __restrict__ rho, const double* __restrict__ ux,
                                 const double* __restrict__ uy, const double* __restrict__ uz,
                                 const double* __restrict__ T, int nx, int ny, int nz, double G,
                                 int psi_kind, double va, double vb, double vT,
-                                double* __restrict__ out /* [nz][3] */) {
-  __shared__ double sh[32];
-  const int z = blockIdx.x;
+                                double* __restrict__ out /* [nz][np][3] */) {
+  __shared__ double sh[4][kThreads];
+  const int z = (int)blockIdx.x / np, part = (int)blockIdx.x - z * np;
   const int nxy = nx * ny;
   const size_t base = (size_t)z * nxy;
   double sr = 0.0, sT = 0.0, sPD = 0.0;
-  for (int i = threadIdx.x; i < nxy; i += blockDim.x) {
+  for (int i = part * kThreads + (int)threadIdx.x; i < nxy; i += np * kThreads) {
     const int x = i % nx, y = i / nx;
     const size_t k = base + i;
+    const int xm = x == 0 ? nx - 1 : x - 1, xp = x + 1 == nx ? 0 : x + 1;
+    const int ym = y == 0 ? ny - 1 : y - 1, yp = y + 1 == ny ? 0 : y + 1;
     const double r = rho[k], t = T[k];
     const double uzp = (z + 1 < nz) ? uz[k + nxy] : -uz[k];
     const double uzm = (z - 1 >= 0) ? uz[k - nxy] : -uz[k];
-    const double D = 0.5 * (ux[base + y * nx + (x + 1) % nx] - ux[base + y * nx + (x + nx - 1) % nx]) +
-                     0.5 * (uy[base + ((y + 1) % ny) * nx + x] - uy[base + ((y + ny - 1) % ny) * nx + x]) +
-                     0.5 * (uzp - uzm);
+    const double D = 0.5 * (((ux[base + y * nx + xp] - ux[base + y * nx + xm]) +
+                             (uy[base + (size_t)yp * nx + x] - uy[base + (size_t)ym * nx + x])) + (uzp - uzm));
     const double P = r * t + ((psi_kind == PSI_VDW) ? r * r * (vb * vT / (1.0 - vb * r) - va)
                                                     : 0.5 * G * exp(-2.0 / r));
     sr += r; sT += t; sPD += P * D;
   }
-  const double a = block_sum(sr, sh), b = block_sum(sT, sh), c = block_sum(sPD, sh);
-  if (threadIdx.x == 0) {
-    out[3 * z] = a / nxy; out[3 * z + 1] = b / nxy; out[3 * z + 2] = c / nxy;
-  }
+  const double v[4] = {sr, sT, sPD, 0.0};
+  const double a = block_sum4(v, sh);
+  const int w = threadIdx.x >> 5;
+  if ((threadIdx.x & 31) == 0 && w < 3) out[3 * (size_t)blockIdx.x + w] = a / nxy;
 }
 
 // Joint histogram of (T, rho) over planes [z_lo, z_hi): bin = floor((v - lo)/(hi - lo) * n) for
@@ -84,33 +104,38 @@ __global__ void histogram_kernel(const double* __restrict__ rho, const double* _
 }
 
 // Structure functions for horizontal increments: block (r-1, z - z_lo) sums over plane z of
-// (q(x + r e_x) - q(x))^p + (q(x + r e_y) - q(x))^p for q = u_z, T and p = 2, 4.
+// (q(x + r e_x) - q(x))^p + (q(x + r e_y) - q(x))^p for q = u_z, T and p = 2, 4. Bound by its 16 FP64
+// instructions per node and r (96^2 x 72 nodes, r <= 32: 0.54 ms at the pipe's rate; 0.66 ms, 0.78
+// before the sums went through shared memory and the rows needed no division).
 __global__ void structure_kernel(const double* __restrict__ uz, const double* __restrict__ T,
                                  int nx, int ny, int z_lo, double* __restrict__ out /* [rmax][nzs][4] */,
                                  int nzs) {
-  __shared__ double sh[32];
+  __shared__ double sh[4][kThreads];
   const int r = blockIdx.x + 1;
   const int zi = blockIdx.y;
-  const int z = z_lo + zi;
-  const int nxy = nx * ny;
-  const size_t base = (size_t)z * nxy;
+  const size_t base = (size_t)(z_lo + zi) * nx * ny;
   double a2 = 0.0, a4 = 0.0, b2 = 0.0, b4 = 0.0;
-  for (int i = threadIdx.x; i < nxy; i += blockDim.x) {
-    const int x = i % nx, y = i / nx;
-    const size_t k = base + i;
-    const size_t kx = base + y * nx + (x + r) % nx;
-    const size_t ky = base + ((y + r) % ny) * nx + x;
-    const double du1 = uz[kx] - uz[k], du2 = uz[ky] - uz[k];
-    const double dt1 = T[kx] - T[k], dt2 = T[ky] - T[k];
-    const double du1s = du1 * du1, du2s = du2 * du2, dt1s = dt1 * dt1, dt2s = dt2 * dt2;
-    a2 += du1s + du2s; a4 += du1s * du1s + du2s * du2s;
-    b2 += dt1s + dt2s; b4 += dt1s * dt1s + dt2s * dt2s;
+  auto take = [](double d1, double d2, double& s2, double& s4) {
+    const double p = d1 * d1, q = d2 * d2;
+    s2 += p; s2 += q;
+    s4 = fma(p, p, s4); s4 = fma(q, q, s4);
+  };
+  // a warp per row, its lanes along x
+  for (int y = (int)(threadIdx.x >> 5); y < ny; y += kWarps) {
+    const int yr = y + r < ny ? y + r : y + r - ny;
+    const double *u0 = uz + base + (size_t)y * nx, *ur = uz + base + (size_t)yr * nx;
+    const double *t0 = T + base + (size_t)y * nx, *tr = T + base + (size_t)yr * nx;
+    for (int x = (int)(threadIdx.x & 31); x < nx; x += 32) {
+      const int xr = x + r < nx ? x + r : x + r - nx;
+      const double u = u0[x], t = t0[x];
+      take(u0[xr] - u, ur[x] - u, a2, a4);
+      take(t0[xr] - t, tr[x] - t, b2, b4);
+    }
   }
-  const double s0 = block_sum(a2, sh), s1 = block_sum(a4, sh), s2 = block_sum(b2, sh), s3 = block_sum(b4, sh);
-  if (threadIdx.x == 0) {
-    double* o = out + ((size_t)(r - 1) * nzs + zi) * 4;
-    o[0] = s0; o[1] = s1; o[2] = s2; o[3] = s3;
-  }
+  const double v[4] = {a2, a4, b2, b4};
+  const double s = block_sum4(v, sh);
+  const int w = threadIdx.x >> 5;
+  if ((threadIdx.x & 31) == 0 && w < 4) out[((size_t)(r - 1) * nzs + zi) * 4 + w] = s;
 }
 
 // Local convective heat flux q = rho U u_z, U = c_v T + U_NI(rho) (the bulk term of Nu, Eq. (4)).
@@ -174,14 +199,19 @@ using namespace tlbm;
 
 namespace {
 
-// macroscopic fields of the current state in the context's staging arrays (device)
+// The macroscopic fields asked for (the other pointers null) of the current state in the context's
+// staging arrays (device)
 int fields_on_device(lb_ctx* c, double** rho, double** ux, double** uy, double** uz, double** T) {
   const size_t N = (size_t)c->N;
   if (!c->fields && cudaMalloc(&c->fields, 5 * N * sizeof(double)) != cudaSuccess)
     return lb_fail(c, LB_ENOMEM, "field staging");
-  *rho = c->fields; *ux = c->fields + N; *uy = c->fields + 2 * N; *uz = c->fields + 3 * N;
-  *T = c->fields + 4 * N;
-  return lb_moments(c, *rho, *ux, *uy, *uz, *T, 1);
+  double** out[5] = {rho, ux, uy, uz, T};
+  double* p[5];
+  for (int k = 0; k < 5; ++k) {
+    p[k] = out[k] ? c->fields + k * N : nullptr;
+    if (out[k]) *out[k] = p[k];
+  }
+  return lb_moments(c, p[0], p[1], p[2], p[3], p[4], 1);
 }
 
 struct DevBuf {
@@ -198,18 +228,25 @@ extern "C" int lb_profiles(lb_ctx* c, double* rho_z, double* T_z, double* PdivU_
   if (rc) return rc;
   const int nz = c->p.nz;
   DevBuf out;
-  if (cudaMalloc(&out.p, (size_t)3 * nz * sizeof(double)) != cudaSuccess) return lb_fail(c, LB_ENOMEM, "profiles");
-  ana::profiles_kernel<<<nz, 256, 0, c->stream>>>(rho, ux, uy, uz, T, c->p.nx, c->p.ny, nz, c->p.G,
+  // CTAs per plane: about 2048 nodes each, so that few planes fill the GPU as well
+  const int np = std::max(1, std::min(16, c->plane / 2048));
+  const size_t n = (size_t)3 * nz * np;
+  if (cudaMalloc(&out.p, n * sizeof(double)) != cudaSuccess) return lb_fail(c, LB_ENOMEM, "profiles");
+  ana::profiles_kernel<<<(unsigned)np * (unsigned)nz, ana::kThreads, 0, c->stream>>>(
+      np,rho, ux, uy, uz, T, c->p.nx, c->p.ny, nz, c->p.G,
                                                   c->p.psi_kind, c->p.vdw_a, c->p.vdw_b, c->p.vdw_T,
                                                   static_cast<double*>(out.p));
   LB_CU(c, cudaGetLastError());
-  std::vector<double> h((size_t)3 * nz);
+  std::vector<double> h(n);
   LB_CU(c, cudaMemcpyAsync(h.data(), out.p, h.size() * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
   LB_CU(c, cudaStreamSynchronize(c->stream));
   for (int z = 0; z < nz; ++z) {
-    if (rho_z) rho_z[z] = h[3 * z];
-    if (T_z) T_z[z] = h[3 * z + 1];
-    if (PdivU_z) PdivU_z[z] = h[3 * z + 2];
+    double s[3] = {0.0, 0.0, 0.0};
+    for (int q = 0; q < np; ++q)
+      for (int k = 0; k < 3; ++k) s[k] += h[3 * ((size_t)z * np + q) + k];
+    if (rho_z) rho_z[z] = s[0];
+    if (T_z) T_z[z] = s[1];
+    if (PdivU_z) PdivU_z[z] = s[2];
   }
   return LB_OK;
 }
@@ -220,8 +257,8 @@ extern "C" int lb_histogram_T_rho(lb_ctx* c, int z_lo, int z_hi, int nT, double 
   if (z_lo < 0 || z_hi > c->p.nz || z_lo >= z_hi || nT < 1 || nrho < 1 || (long long)nT * nrho > 12288 ||
       !(T_hi > T_lo) || !(rho_hi > rho_lo))
     return lb_fail(c, LB_EINVAL, "histogram ranges");
-  double *rho, *ux, *uy, *uz, *T;
-  int rc = fields_on_device(c, &rho, &ux, &uy, &uz, &T);
+  double *rho, *T;
+  int rc = fields_on_device(c, &rho, nullptr, nullptr, nullptr, &T);
   if (rc) return rc;
   const int nb = nT * nrho;
   DevBuf cnt;
@@ -242,14 +279,14 @@ extern "C" int lb_structure_functions(lb_ctx* c, int rmax, int z_lo, int z_hi, d
   if (!c) return LB_EINVAL;
   if (rmax < 1 || rmax >= c->p.nx || rmax >= c->p.ny || z_lo < 0 || z_hi > c->p.nz || z_lo >= z_hi)
     return lb_fail(c, LB_EINVAL, "structure-function ranges");
-  double *rho, *ux, *uy, *uz, *T;
-  int rc = fields_on_device(c, &rho, &ux, &uy, &uz, &T);
+  double *uz, *T;
+  int rc = fields_on_device(c, nullptr, nullptr, nullptr, &uz, &T);
   if (rc) return rc;
   const int nzs = z_hi - z_lo;
   DevBuf out;
   const size_t n = (size_t)rmax * nzs * 4;
   if (cudaMalloc(&out.p, n * sizeof(double)) != cudaSuccess) return lb_fail(c, LB_ENOMEM, "structure functions");
-  ana::structure_kernel<<<dim3(rmax, nzs), 256, 0, c->stream>>>(uz, T, c->p.nx, c->p.ny, z_lo,
+  ana::structure_kernel<<<dim3(rmax, nzs), ana::kThreads, 0, c->stream>>>(uz, T, c->p.nx, c->p.ny, z_lo,
                                                                 static_cast<double*>(out.p), nzs);
   LB_CU(c, cudaGetLastError());
   std::vector<double> h(n);
@@ -273,8 +310,8 @@ extern "C" int lb_heat_flux_pdf(lb_ctx* c, int z_lo, int z_hi, int nbins, double
   if (!c) return LB_EINVAL;
   if (z_lo < 0 || z_hi > c->p.nz || z_lo >= z_hi || nbins < 1 || nbins > 12288 || !(q_hi > q_lo))
     return lb_fail(c, LB_EINVAL, "heat-flux pdf ranges");
-  double *rho, *ux, *uy, *uz, *T;
-  int rc = fields_on_device(c, &rho, &ux, &uy, &uz, &T);
+  double *rho, *uz, *T;
+  int rc = fields_on_device(c, &rho, nullptr, nullptr, &uz, &T);
   if (rc) return rc;
   const int blocks = 304;
   DevBuf cnt, part;
