@@ -80,16 +80,18 @@ __global__ void __launch_bounds__(1024) lb_diag_finalize(int nz, int nxy, double
     red[4][warp] = mr; red[5][warp] = mT;
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double a[6] = {red[0][0], red[1][0], red[2][0], red[3][0], red[4][0], red[5][0]};
-    for (int w = 1; w < nwarp; ++w) {
-      for (int k = 0; k < 4; ++k) a[k] += red[k][w];
-      a[4] = fmin(a[4], red[4][w]); a[5] = fmin(a[5], red[5][w]);
+  if (warp == 0) {
+    // the warps' values over the lanes of one warp (a serial chain of 6 x 32 FP64 additions took 15 us)
+    const bool on = lane < nwarp;
+    const double a0 = warp_sum(on ? red[0][lane] : 0.0), a1 = warp_sum(on ? red[1][lane] : 0.0);
+    const double a2 = warp_sum(on ? red[2][lane] : 0.0), a3 = warp_sum(on ? red[3][lane] : 0.0);
+    const double a4 = warp_min(on ? red[4][lane] : 1e300), a5 = warp_min(on ? red[5][lane] : 1e300);
+    if (lane == 0) {
+      const double mean = a0 / nz;
+      out[nz] = mean; out[nz + 1] = a4; out[nz + 2] = a5; out[nz + 3] = a3;
+      out[nz + 4] = a1; out[nz + 5] = a2;
+      if (acc) { acc[0] += mean; acc[1] += 1.0; }
     }
-    const double mean = a[0] / nz;
-    out[nz] = mean; out[nz + 1] = a[4]; out[nz + 2] = a[5]; out[nz + 3] = a[3];
-    out[nz + 4] = a[1]; out[nz + 5] = a[2];
-    if (acc) { acc[0] += mean; acc[1] += 1.0; }
   }
 }
 
@@ -181,16 +183,36 @@ KArgs make_args(const lb_ctx* c) {
   a.pf.irho0 = (float)a.pd.irho0;
   auto split_consts = [&](auto& k) {
     using R = std::decay_t<decltype(k.om1)>;
-    const double wc[3] = {1.0 / 3.0, 1.0 / 18.0, 1.0 / 36.0};
-    k.om1 = (R)(1.0 - a.omega_nu); k.omk1 = (R)(1.0 - a.omega_kappa);
-    for (int q = 0; q < 3; ++q) {
-      k.fo[q] = (R)(wc[q] * a.omega_nu); k.fs[q] = (R)(3.0 * wc[q] * a.omega_nu); k.fq[q] = (R)(4.5 * wc[q] * a.omega_nu);
-      k.go[q] = (R)(wc[q] * a.omega_kappa); k.gs[q] = (R)(3.0 * wc[q] * a.omega_kappa); k.gq[q] = (R)(4.5 * wc[q] * a.omega_kappa);
-    }
-    k.mg = (R)(-a.G / 12.0); k.gz_u = (R)(0.5 * a.g_z); k.gz_v = (R)(a.tau_nu * a.g_z);
-    k.src = (R)(0.5 / (c->p.c_v * a.omega_kappa)); k.lam45 = (R)(4.5 * a.lam);
-    k.v_u = (R)(2.0 * a.tau_nu); k.v_j = (R)(1.0 - 2.0 * a.tau_nu);
-    k.ks = (R)(1.0 - 0.5 * a.omega_nu);
+    constexpr bool F32 = sizeof(R) == 4;
+    // x as R and, for FP32, its remainder
+    auto two = [](double x, R& hi, R& lo) { hi = (R)x; lo = (R)(x - (double)hi); };
+    // the weights of relaxation rate omega; returns the rate that they add up to
+    auto weights = [](double omega, R& om1, R (&o)[3], R (&s3)[3], R (&q)[3]) -> double {
+      double w2 = omega / 36.0;
+      if (F32) {
+        int e;
+        const double m = std::frexp(w2, &e);
+        w2 = std::ldexp(std::nearbyint(std::ldexp(m, 20)), e - 20);
+      }
+      om1 = (R)(1.0 - 36.0 * w2);
+      o[0] = (R)(12.0 * w2); o[1] = (R)(2.0 * w2); o[2] = (R)w2;
+      for (int c = 0; c < 3; ++c) { s3[c] = (R)(3.0 * (double)o[c]); q[c] = (R)(4.5 * (double)o[c]); }
+      return F32 ? 36.0 * w2 : omega;
+    };
+    const double en = weights(a.omega_nu, k.om1, k.fo, k.fs, k.fq);
+    const double ek = weights(a.omega_kappa, k.omk1, k.go, k.gs, k.gq);
+    const double tau = F32 ? 1.0 / en : a.tau_nu;      // so that a step adds F to j, whole
+    const bool dev = F32 && a.psi_kind != PSI_VDW;
+    // the reference density of the FP32 forms is the rounded one (their deviations are from it)
+    const double r0 = (double)k.rho0, p0 = std::exp(-1.0 / r0);
+    two(dev ? -a.G * p0 * p0 / 12.0 : -a.G / 12.0, k.mg, k.mg_lo);
+    R hi;
+    two(1.0 / r0, hi, k.irho0_lo);
+    k.irho0 = hi;
+    two(tau, k.tau, k.tau_lo);
+    k.gz_u = (R)(0.5 * a.g_z); k.gz_v = (R)(tau * a.g_z);
+    k.src = (R)(0.5 / (c->p.c_v * ek)); k.lam45 = (R)(4.5 * a.lam);
+    k.ks = (R)(1.0 - 0.5 * en);
   };
   split_consts(a.pd);
   split_consts(a.pf);
@@ -268,7 +290,8 @@ void free_all(lb_ctx* c) {
 // Nu_mean is added to acc[0] (and 1 to acc[1]) when acc is not null.
 int finalize_diag(lb_ctx* c, double* acc) {
   lb_diag_planes<<<c->p.nz, 128, 0, c->stream>>>(c->part, c->p.nz, c->nblk, c->diag);
-  lb_diag_finalize<<<1, 1024, 0, c->stream>>>(c->p.nz, c->p.nx * c->p.ny, c->p.kappa, c->p.T_d,
+  const int ft = std::min(1024, (c->p.nz + 31) / 32 * 32);
+  lb_diag_finalize<<<1, ft, 0, c->stream>>>(c->p.nz, c->p.nx * c->p.ny, c->p.kappa, c->p.T_d,
                                                c->p.T_u, c->diag, acc);
   LB_CU(c, cudaGetLastError());
   return LB_OK;

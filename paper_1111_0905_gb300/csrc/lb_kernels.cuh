@@ -123,11 +123,17 @@ template <class R> struct KPar {
   R tau_nu, omega_nu, omega_kappa, G, g_z, lam, inv_cv, T_d, T_u, rho0, T0, E0;
   R va, vb, vT, vk;   // van der Waals-type psi: a, b, T_v, 2/(-G)
   R psi0, irho0;      // psi(rho0) = exp(-1/rho0) and 1/rho0 (deviation form of psi)
-  // three-kernel step: 1 - omega and, per class (rest, axis, diagonal), w omega, 3 w omega, 4.5 w omega
+  // Constants of lb_split.cuh and lb_march.cuh. The force and the ideal pressure nearly cancel in the
+  // flows of interest, so a relative rounding of 6e-8 in any one factor of either shows as a velocity
+  // error that is the same everywhere and adds up over the steps. In FP32 therefore the factors of F
+  // carry their rounding as a second float (_lo), and the weights per class (rest, axis, diagonal:
+  // w om, 3 w om, 4.5 w om) and 1 - om are exact multiples of one number (w om of a diagonal, rounded
+  // to 20 bits), so that mass, momentum and pressure relax consistently.
   R om1, omk1, fo[3], fs[3], fq[3], go[3], gs[3], gq[3];
-  R mg, gz_u, gz_v;   // -G/12; g_z/2 and tau g_z
+  R mg, mg_lo;        // -G/12 (FP32, the paper's psi: -G psi(rho0)^2/12)
+  R irho0_lo, tau, tau_lo;   // tau = 1/(36 w om)
+  R gz_u, gz_v;       // g_z/2 and tau g_z
   R src, lam45;       // 1/(2 c_v omega_kappa), 4.5 lam
-  R v_u, v_j;         // u' = v_u u + v_j j/rho: 2 tau and 1 - 2 tau
   R ks;               // 1 - omega_nu/2 (Guo forcing)
 };
 

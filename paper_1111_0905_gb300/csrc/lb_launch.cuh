@@ -152,7 +152,9 @@ template <class S> struct OpsImpl {
     const unsigned grid = (unsigned)nb * (unsigned)a.nz;
     cudaError_t e;
     if ((e = follow(split_moments_kernel<S, (VAR & VAR_VDW) != 0, NT>, grid, NT, st, a, nb)) != cudaSuccess) return e;
-    if ((e = follow(split_velocity_kernel<R, VAR, NT>, grid, NT, st, a, nb)) != cudaSuccess) return e;
+    if (mode != MODE_MOMENTS || wants_velocity(a)) {
+      if ((e = follow(split_velocity_kernel<R, VAR, NT>, grid, NT, st, a, nb)) != cudaSuccess) return e;
+    }
     if (mode == MODE_STEP) return follow(split_collide_kernel<S, VAR, MODE_STEP, NT>, grid, NT, st, a, nb);
     if (mode == MODE_MOMENTS) return follow(split_collide_kernel<S, VAR & VAR_VDW, MODE_MOMENTS, NT>, grid, NT, st, a, nb);
     // the fused step + Nu sample exists for the paper's scheme only (the caller checks)

@@ -109,18 +109,30 @@ __device__ __forceinline__ void pair_gradient(const R (&d)[Q / 2], R& ax, R& ay,
   az = R(2) * d[2] + ((d[5] - d[6]) + (d[7] - d[8]));
 }
 
-// psi of a node as the fields keep it (FP32 compute, the paper's psi: its deviation from psi(rho0))
+// psi of a node as the fields keep it. FP32 compute, the paper's psi: e = psi/psi(rho0) - 1 = e^t - 1,
+// t = 1/rho0 - 1/rho = drho/(rho rho0) (sum_l W_l c_l = 0, so the force sum may take e for psi; it then
+// adds small numbers).
 template <class R, bool VDW>
 __device__ __forceinline__ R split_psi(R rho, R drho, R inv, const KPar<R>& kp) {
   if constexpr (VDW) return psi_vdw(rho, kp);
   else if constexpr (sizeof(R) == 8) return fexp(-inv);
-  else return kp.psi0 * expm1_dev(drho * inv * kp.irho0);
+  else {
+    const R x = drho * inv;
+    return expm1_dev(fma_rn(x, kp.irho0, x * kp.irho0_lo));
+  }
 }
-// -G psi / 12 from psi as kept
+// -G psi / 12 (FP32 compute, the paper's psi: times psi(rho0)) from psi as kept
 template <class R, bool VDW>
 __device__ __forceinline__ R split_mg(R psi, const KPar<R>& kp) {
-  return kp.mg * ((sizeof(R) == 4 && !VDW) ? kp.psi0 + psi : psi);
+  if constexpr (sizeof(R) == 8) return kp.mg * psi;
+  else {
+    const R p = VDW ? psi : R(1) + psi;
+    return fma_rn(kp.mg, p, kp.mg_lo * p);
+  }
 }
+// tau F-factor / rho from F-factor / rho
+__device__ __forceinline__ double split_mv(double mi, const KPar<double>& kp) { return kp.tau * mi; }
+__device__ __forceinline__ float split_mv(float mi, const KPar<float>& kp) { return fma_rn(kp.tau, mi, kp.tau_lo * mi); }
 
 // BGK relaxation of one lattice towards its equilibrium around the velocity v, pair by pair:
 //   out_l = om1 in_l + [ev + 9 (c.v)(c.F')] +- [s (c.v) + 3 (c.F')],  ev = q (c.v)^2 + P per class,
@@ -192,23 +204,46 @@ template <class R> struct DiagTerms {
     T = t; rho = r; E = e; mr = r; mT = t;
     bad = !(isfinite(r) && isfinite(t) && isfinite(ux) && isfinite(uy) && isfinite(uz));
   }
-  // warp sums in the compute precision into red[7][NW] (column w)
+  // Warp sums in the compute precision into red[7][NW] (column w). The four sums are reduced together,
+  // each exchange halving the values a lane carries (6 shuffles instead of 20), the two minima likewise.
   template <int NW> __device__ __forceinline__ void reduce(R (&red)[7][NW], int w, int lane) {
-    conv = warp_sum(conv); T = warp_sum(T); rho = warp_sum(rho); E = warp_sum(E);
-    mr = warp_min(mr); mT = warp_min(mT);
-    const int nbad = __popc(__ballot_sync(0xffffffffu, bad));
-    if (lane == 0) {
-      red[0][w] = conv; red[1][w] = T; red[2][w] = rho; red[3][w] = E; red[4][w] = mr; red[5][w] = mT;
-      red[6][w] = R(nbad);
+    const bool hi = (lane & 16) != 0, mid = (lane & 8) != 0;
+    const R p = (hi ? rho : conv) + __shfl_xor_sync(0xffffffffu, hi ? conv : rho, 16);
+    const R q = (hi ? E : T) + __shfl_xor_sync(0xffffffffu, hi ? T : E, 16);
+    R s = (mid ? q : p) + __shfl_xor_sync(0xffffffffu, mid ? p : q, 8);
+    R m = fmin(hi ? mT : mr, __shfl_xor_sync(0xffffffffu, hi ? mr : mT, 16));
+    m = fmin(m, __shfl_xor_sync(0xffffffffu, m, 8));
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) {
+      s += __shfl_xor_sync(0xffffffffu, s, o);
+      m = fmin(m, __shfl_xor_sync(0xffffffffu, m, o));
     }
+    const int nbad = __popc(__ballot_sync(0xffffffffu, bad));
+    // lanes 0, 8, 16, 24 hold conv, T, rho, E; lanes 0 and 16 the minima
+    if ((lane & 7) == 0) red[lane >> 3][w] = s;
+    if ((lane & 15) == 0) red[4 + (lane >> 4)][w] = m;
+    if (lane == 0) red[6][w] = R(nbad);
   }
 };
-// partial q of one CTA's plane piece, over its warps in order, in FP64
+// The partials of one CTA's plane piece from its warps', by one warp: eight lanes per quantity, the sums
+// in FP64 in a fixed tree (a chain over the warps took twice as long).
 template <class R, int NW>
-__device__ __forceinline__ void diag_combine(const R (&red)[7][NW], int q, double* part) {
-  double acc = double(red[q][0]);
-  for (int k = 1; k < NW; ++k) acc = (q == 4 || q == 5) ? fmin(acc, double(red[q][k])) : acc + double(red[q][k]);
-  part[q] = acc;
+__device__ __forceinline__ void diag_combine(const R (&red)[7][NW], int lane, double* part) {
+  static_assert(NW <= 8, "eight lanes per quantity");
+  const int k = lane >> 3, w = lane & 7;
+  double s = w < NW ? double(red[k][w]) : 0.0;                       // conv, T, rho, E
+  const int km = 4 + (k < 2 ? k : 2);                                // min rho, min T, non-finite
+  R m = w < NW ? red[km][w] : (km == 6 ? R(0) : R(sizeof(R) == 8 ? 1e300 : 3.0e38));
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) {
+    s += __shfl_xor_sync(0xffffffffu, s, o);
+    const R n = __shfl_xor_sync(0xffffffffu, m, o);
+    m = km == 6 ? m + n : fmin(m, n);
+  }
+  if (w == 0) {
+    part[k] = s;
+    if (k < 3) part[4 + k] = double(m);
+  }
 }
 
 // The kernels of one step follow each other closely: each is launched as its predecessor's CTAs end
@@ -276,7 +311,7 @@ __global__ void __launch_bounds__(NT) split_velocity_kernel(const KArgs a, int n
   else inv = recip(rho);
   const R mg = split_mg<R, VDW>(ld_at(p0, n.i), kp);              // F = mg A + rho g_z z
   const R mi = mg * inv;
-  const R mu = R(0.5) * mi, mv = kp.tau_nu * mi;
+  const R mu = R(0.5) * mi, mv = split_mv(mi, kp);
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
     const R j = ld_at(static_cast<const R*>(a.fd_j[k]) + zo, n.i);
@@ -297,12 +332,20 @@ __global__ void __launch_bounds__(NT) split_velocity_kernel(const KArgs a, int n
 
 // Resident 256-thread CTAs per SM that the collision's registers allow. FP32: 64 registers (4 CTAs;
 // 256^3 boiling cell 0.84 ms against 0.90 with 3 and 0.97 with 2); 16-bit 80 (3); FP64 128 (2).
-template <class S> constexpr int split_mb() { return sizeof(S) == 4 ? 4 : (sizeof(S) == 2 ? 3 : 2); }
+template <class S, int MODE> constexpr int split_mb() {
+  if (MODE == MODE_MOMENTS) return sizeof(S) == 8 ? 3 : 4;    // holds one lattice only
+  return sizeof(S) == 4 ? 4 : (sizeof(S) == 2 ? 3 : 2);
+}
+
+// whether a moments pass needs the velocities (an exported component or the diagnostics)
+__host__ __device__ __forceinline__ bool wants_velocity(const KArgs& a) {
+  return a.ux_out || a.uy_out || a.uz_out || a.part;
+}
 
 // MODE_MOMENTS: the fields of the state read instead of the collision; DIAG modes: the partials of
 // the state read, one set per CTA.
 template <class S, int VAR, int MODE, int NT>
-__global__ void __launch_bounds__(NT, split_mb<S>() * 256 / NT) split_collide_kernel(const KArgs a, int nb) {
+__global__ void __launch_bounds__(NT, split_mb<S, MODE>() * 256 / NT) split_collide_kernel(const KArgs a, int nb) {
   using R = typename Store<S>::R;
   constexpr bool GUO = (VAR & VAR_GUO) != 0, VDW = (VAR & VAR_VDW) != 0, F64 = sizeof(R) == 8;
   constexpr bool COLLIDE = MODE != MODE_MOMENTS, DIAG = MODE != MODE_STEP;
@@ -326,7 +369,9 @@ __global__ void __launch_bounds__(NT, split_mb<S>() * 256 / NT) split_collide_ke
     const R* puy = static_cast<const R*>(a.fd_u[1]) + zo;
     const R* puz = static_cast<const R*>(a.fd_u[2]) + zo;
     const R rv = ld_at(static_cast<const R*>(a.fd_rho) + zo, o);
-    const R ux = ld_at(pux, o), uy = ld_at(puy, o), uz = ld_at(puz, o);
+    // a moments pass that asks for rho and T only has no velocities formed
+    const bool need_u = COLLIDE || wants_velocity(a);
+    const R ux = need_u ? ld_at(pux, o) : R(0), uy = need_u ? ld_at(puy, o) : R(0), uz = need_u ? ld_at(puz, o) : R(0);
     R inv;
     if constexpr (F64) inv = ld_at(static_cast<const R*>(a.fd_inv) + zo, o);
     if (z == 0 || z == a.nz - 1)
@@ -339,7 +384,9 @@ __global__ void __launch_bounds__(NT, split_mb<S>() * 256 / NT) split_collide_ke
     for (int l = 1; l < Q; ++l) dE = dE + g[l];
     const R E = kp.E0 + dE;
     const R T = E * inv;            // the plain step needs it for the adjoint's fields only
-    if constexpr (DIAG) dt.template take<VDW>(a, rho, inv, T, E, ux, uy, uz);
+    if constexpr (DIAG) {
+      if (a.part != nullptr) dt.template take<VDW>(a, rho, inv, T, E, ux, uy, uz);
+    }
     if constexpr (COLLIDE) {
       const R uzp = z + 1 < a.nz ? ld_at(puz + plane, o) : -uz;
       const R uzm = z > 0 ? ld_at(puz - plane, o) : -uz;
@@ -356,9 +403,11 @@ __global__ void __launch_bounds__(NT, split_mb<S>() * 256 / NT) split_collide_ke
         R dr, j[3];
         pair_moments<R>(f, dr, j[0], j[1], j[2]);
         const R u[3] = {ux, uy, uz};
-        const R c = inv * kp.v_j;           // (1 - 2 tau)/rho
 #pragma unroll
-        for (int k = 0; k < 3; ++k) w[k] = GUO ? R(2) * (rho * u[k] - j[k]) : kp.v_u * u[k] + c * j[k];
+        for (int k = 0; k < 3; ++k) {
+          const R ji = j[k] * inv;
+          w[k] = GUO ? R(2) * (rho * u[k] - j[k]) : ji + split_mv(R(2) * (u[k] - ji), kp);   // u - j/rho = F/(2 rho)
+        }
       }
       S* __restrict__ fo = static_cast<S*>(a.fout) + zo;
       S* __restrict__ go = static_cast<S*>(a.gout) + zo;
@@ -396,7 +445,7 @@ __global__ void __launch_bounds__(NT, split_mb<S>() * 256 / NT) split_collide_ke
       __shared__ R red[7][NW];
       dt.template reduce<NW>(red, threadIdx.x >> 5, threadIdx.x & 31);
       __syncthreads();
-      if (threadIdx.x < 7) diag_combine<R, NW>(red, (int)threadIdx.x, a.part + (size_t)blockIdx.x * NPART);
+      if (threadIdx.x < 32) diag_combine<R, NW>(red, (int)threadIdx.x, a.part + (size_t)blockIdx.x * NPART);
     }
   }
 }
