@@ -243,10 +243,11 @@ namespace {
 // nodes. (256^3: 8.9 ms against 10.7 with the tile march and its pre-pass.)
 //
 // FP32 compute takes the one-launch march, unless three kernels are expected to be faster. A march
-// iteration (one plane of a CTA) takes about 1.8 us and a CTA of zc planes zc + 4 of them and about
-// two more to start, one CTA per SM, in waves: ceil(CTAs / SMs) (zc + 6) iterations. The three
-// kernels take about 12 us and 78 ps per node (FP32: 128^3 168 us, 64^3 28 us, 32^3 15 us; march
-// 128^3 126 us). The chunk zc is the one of the least cost.
+// iteration is one plane of a CTA; a CTA of zc planes takes zc + 4 of them and about two more to
+// start, one CTA per SM, in waves: ceil(CTAs / SMs) (zc + 6) iterations. Measured per iteration (128^3,
+// 256^3): FP32 1.8 us, 16-bit deviations 1.5 us, local references 2.2 us. The three kernels take about
+// 7 us and per node 73, 58 and 77 ps (FP32 64^3 28 us and 128^3 168 us, the march 21 and 126 us; 32^3
+// 7.6 us against 18; local references 96^3 72 us against 86). The chunk zc is the one of the least cost.
 cudaError_t choose_form(lb_ctx* c) {
   c->nblk = c->ntiles;
   if (c->p.tile_y != 0 || c->p.z_chunk != 0) { c->form = lb_ctx::kTile; return cudaSuccess; }
@@ -265,7 +266,9 @@ cudaError_t choose_form(lb_ctx* c) {
       const long long cost = ((ctas + sms - 1) / sms) * (zc + 6);
       if (best < 0 || cost < best) { best = cost; c->march_zc = zc; }
     }
-    if (1.8e-6 * (double)best < 12e-6 + 78e-12 * (double)c->N) {
+    const bool b16 = c->ops->esize == 2, loc = c->ops->slots > Q;
+    const double iteration = loc ? 2.2e-6 : (b16 ? 1.5e-6 : 1.8e-6), node = loc ? 77e-12 : (b16 ? 58e-12 : 73e-12);
+    if (iteration * (double)best < 7e-6 + node * (double)c->N) {
       c->form = lb_ctx::kMarch;
       c->nblk = (int)tiles;
       return cudaSuccess;

@@ -175,10 +175,10 @@ template <class S> struct OpsImpl {
 
   // The one-launch step (lb_march.cuh). Tile heights: measured on the 256^3 and 512^3 boiling cells,
   // FP32 7, 8, 9, 10, 12 rows: 0.99, 0.95, 1.03, 1.05, 1.13 ms and 8.0, 7.5, 7.3, 7.9, 8.5 ms; FP16
-  // deviations 7, 8, 9, 12 rows: 0.78, 0.72, 0.80, 0.95 ms at 256^3; local references 4, 5, 6, 7, 8
-  // rows: 1.27, 1.24, 1.86, 1.5, 1.80 ms (their 39 values in flight per thread spill beyond 5). Taller
-  // tiles recompute fewer ring nodes but leave fewer registers per thread.
-  static constexpr int MTY = IsLoc<S>::v ? 5 : 8;
+  // deviations 7, 8, 9, 12 rows: 0.78, 0.72, 0.80, 0.95 ms at 256^3; local references 5, 6, 7, 8 rows:
+  // 1.30, 1.34, 1.18, 1.42 ms. Taller tiles recompute fewer ring nodes but leave fewer registers per
+  // thread, and a spilled value in flight makes its warp wait for it.
+  static constexpr int MTY = IsLoc<S>::v ? 7 : 8;
   template <int VAR, int MODE> static cudaError_t march_go(const KArgs& a, const MarchArgs& b, dim3 grid, cudaStream_t st) {
     using GE = MarchGeo<S, MTY>;
     split_march_kernel<S, VAR, MODE, MTY><<<grid, GE::NT, GE::smem, st>>>(a, b);
@@ -213,14 +213,14 @@ template <class S> struct OpsImpl {
         b.gdst[l] = static_cast<char*>(a.gout) + l * N * es;
       }
       for (int l = 0; l < Q; ++l) {
-        const long long src = (l * N - CZ(l) * plane) * es, ref = ((l == 0 ? Q : Q - 1 + CSQ(l)) * N - CZ(l) * plane) * es;
+        const long long src = (l * N - CZ(l) * plane) * es;
         b.fsrc[l] = static_cast<const char*>(a.fin) + src;
         b.gsrc[l] = static_cast<const char*>(a.gin) + src;
-        b.fref[l] = static_cast<const char*>(a.fin) + ref;
-        b.gref[l] = static_cast<const char*>(a.gin) + ref;
       }
-      b.fref[Q] = static_cast<const char*>(a.fin) + (Q + 1) * N * es;
-      b.gref[Q] = static_cast<const char*>(a.gin) + (Q + 1) * N * es;
+      for (int k = 0; k < 2; ++k) {
+        b.fref[k] = static_cast<const char*>(a.fin) + (Q + k) * N * es;
+        b.gref[k] = static_cast<const char*>(a.gin) + (Q + k) * N * es;
+      }
       b.tiles_x = (a.nx + BX - 1) / BX;
       b.zc = zc;
       const dim3 grid((unsigned)(b.tiles_x * ((a.ny + MTY - 1) / MTY)), (unsigned)((a.nz + zc - 1) / zc));

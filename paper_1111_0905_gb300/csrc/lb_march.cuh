@@ -13,13 +13,12 @@
 namespace tlbm {
 
 // Where the populations are read and written, as bytes: per population the start of its lattice
-// plane -c_lz relative to the node's own plane (pull source) and of its lattice (store); with the
-// local references likewise the reference slot that belongs to the source of population l (entry 0:
-// slot 19 of the node itself, entry 19: slot 20 of the node itself).
+// plane -c_lz relative to the node's own plane (pull source) and of its lattice (store). The local
+// references are slots 19 and 20 of either lattice, read from fdst's counterparts fref and gref.
 struct MarchArgs {
   const char* fsrc[Q]; const char* gsrc[Q];
   char* fdst[Q + 2]; char* gdst[Q + 2];
-  const char* fref[Q + 1]; const char* gref[Q + 1];
+  const char* fref[2]; const char* gref[2];
   int tiles_x, zc;
 };
 
@@ -29,7 +28,10 @@ template <class S, int TY> struct MarchGeo {
   static constexpr int DF = 4;   // planes of f kept: C of plane p-2 may still run when M writes plane p+1
   // psi [4][NM], ux, uy [3][2][NM], u', drho, 1/rho [3][5][NC], uz [3][NC], f [DF][Q][NC]
   static constexpr size_t floats = 4 * NM + 6 * NM + 15 * NC + 3 * NC;
-  static constexpr size_t smem = 4 * floats + sizeof(FC) * DF * Q * NC;
+  // local references: windows of four planes of 4-byte words (slot 19 low, slot 20 high half), of f on the ring's
+  // neighbourhood (radius 3 of the tile), of g on the tile's (radius 1)
+  static constexpr int FWX = 38, FW = FWX * (TY + 6), GWX = 34, GW = GWX * (TY + 2);
+  static constexpr size_t smem = 4 * floats + sizeof(FC) * DF * Q * NC + (IsLoc<S>::v ? 16 * (FW + GW) : 0);
 };
 
 __device__ __forceinline__ void bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
@@ -66,23 +68,14 @@ __device__ __forceinline__ __half ld_here(const char* p, __half) { return __usho
 __device__ __forceinline__ __nv_bfloat16 ld_here(const char* p, __nv_bfloat16) { return __ushort_as_bfloat16(ld_here16(p)); }
 __device__ __forceinline__ half_loc ld_here(const char* p, half_loc) { half_loc h; h.h = __ushort_as_half(ld_here16(p)); return h; }
 
-// The stored values that a node pulls, in flight or arrived (with their references)
+// The stored values that a node pulls, in flight or arrived
 template <class S> struct MarchRaw {
-  static constexpr int NREF = IsLoc<S>::v ? Q + 1 : 1;
   S v[Q];
-  S r[NREF];
   // request the node at m of plane z
-  __device__ __forceinline__ void request(const char* const (&src)[Q], const char* const (&ref)[Q + 1], const KArgs& a,
-                                          int z, const MarchPos<S>& m) {
+  __device__ __forceinline__ void request(const char* const (&src)[Q], const KArgs& a, int z, const MarchPos<S>& m) {
     if (z > 0 && z < a.nz - 1) {
 #pragma unroll
       for (int l = 0; l < Q; ++l) v[l] = ld_here(src[l] + (size_t)m.v[1 - CX(l)][1 - CY(l)], S());
-      if constexpr (IsLoc<S>::v) {
-        r[0] = ld_here(ref[0] + (size_t)m.v[1][1], S());
-        r[Q] = ld_here(ref[Q] + (size_t)m.v[1][1], S());
-#pragma unroll
-        for (int l = 1; l < Q; ++l) r[l] = ld_here(ref[l] + (size_t)m.v[1 - CX(l)][1 - CY(l)], S());
-      }
     } else {
       // through a wall: the bounce-back source, population opp(l) of the node itself
       const long long pb = (long long)a.plane * (long long)sizeof(S);
@@ -92,26 +85,76 @@ template <class S> struct MarchRaw {
         const char* b = through ? src[OPP(l)] + CZ(OPP(l)) * pb : src[l];
         v[l] = ld_here(b + (size_t)(through ? m.v[1][1] : m.v[1 - CX(l)][1 - CY(l)]), S());
       }
-      if constexpr (IsLoc<S>::v) {
-        r[0] = ld_here(ref[0] + (size_t)m.v[1][1], S());
-        r[Q] = ld_here(ref[Q] + (size_t)m.v[1][1], S());
-#pragma unroll
-        for (int l = 1; l < Q; ++l) {
-          const bool through = (CZ(l) > 0 && z == 0) || (CZ(l) < 0 && z == a.nz - 1);
-          const char* b = through ? ref[l] + CZ(l) * pb : ref[l];
-          r[l] = ld_here(b + (size_t)(through ? m.v[1][1] : m.v[1 - CX(l)][1 - CY(l)]), S());
-        }
-      }
     }
   }
-  __device__ __forceinline__ void decode(float (&f)[Q]) const {
+  // the deviations; with local references from the window word i of plane z (rows of WX words)
+  template <int WX, int WN>
+  __device__ __forceinline__ void decode(float (&f)[Q], const uint32_t* win, int i, int z, int nz) const {
 #pragma unroll
     for (int l = 0; l < Q; ++l) f[l] = cvt<S, float>(v[l]);
     if constexpr (IsLoc<S>::v) {
-      f[0] += 12.0f * (cvt<S, float>(r[0]) - cvt<S, float>(r[Q]));
+      const uint32_t* w0 = win + (z & 3) * WN + i;
+      // a plane beyond a wall: the node's own word (the bounce-back source)
+      const bool bot = z == 0, top = z == nz - 1;
+      const uint32_t* wm = win + ((z - 1) & 3) * WN + i;
+      const uint32_t* wp = win + ((z + 1) & 3) * WN + i;
+      auto lo = [](uint32_t w) { return __half2float(__ushort_as_half((unsigned short)(w & 0xffffu))); };
+      auto hi = [](uint32_t w) { return __half2float(__ushort_as_half((unsigned short)(w >> 16))); };
+      f[0] += 12.0f * (lo(w0[0]) - hi(w0[0]));
 #pragma unroll
-      for (int l = 1; l < Q; ++l) f[l] += cvt<S, float>(r[l]);
+      for (int l = 1; l < Q; ++l) {
+        const int st = -(CY(l) * WX + CX(l));
+        uint32_t w;
+        if (CZ(l) == 0) w = w0[st];
+        else if (CZ(l) > 0) w = bot ? w0[0] : wm[st];
+        else w = top ? w0[0] : wp[st];
+        f[l] += CSQ(l) == 1 ? lo(w) : hi(w);
+      }
     }
+  }
+};
+
+// Feeds a window of references, WX x WN/WX nodes from (x0, y0), by NTH threads (up to two nodes each):
+// the references of a plane are requested an iteration before they are stored.
+template <int WX, int WN, int NTH> struct RefFeed {
+  unsigned off[2];
+  unsigned short a[2], b[2];
+  int t;
+  __device__ __forceinline__ void set(const KArgs& ka, int thread, int x0, int y0) {
+    static_assert(WN <= 2 * NTH, "two words per thread");
+    t = thread;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const int i = t + k * NTH;
+      off[k] = 2u * ((unsigned)wrapi(y0 + i / WX, ka.ny) * (unsigned)ka.nx + (unsigned)wrapi(x0 + i % WX, ka.nx));
+    }
+  }
+  __device__ __forceinline__ void request(const char* const (&ref)[2], size_t plane_bytes, int z) {
+    const char* p0 = ref[0] + (size_t)z * plane_bytes;
+    const char* p1 = ref[1] + (size_t)z * plane_bytes;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      if (t + k * NTH < WN) { a[k] = ld_here16(p0 + off[k]); b[k] = ld_here16(p1 + off[k]); }
+    }
+  }
+  __device__ __forceinline__ void store(uint32_t* win, int z) const {
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const int i = t + k * NTH;
+      if (i < WN) win[(z & 3) * WN + i] = (uint32_t)a[k] | ((uint32_t)b[k] << 16);
+    }
+  }
+  // planes z-1 .. z+1 at once, and z+2 requested
+  __device__ __forceinline__ void start(const char* const (&ref)[2], size_t plane_bytes, uint32_t* win, int z, int nz) {
+    for (int q = z - 1; q <= z + 1; ++q) {
+      if (q >= 0 && q < nz) { request(ref, plane_bytes, q); store(win, q); }
+    }
+    if (z + 2 < nz) request(ref, plane_bytes, z + 2);
+  }
+  // behind the use of planes z-1 .. z+1: plane z+2 into the window, z+3 requested
+  __device__ __forceinline__ void next(const char* const (&ref)[2], size_t plane_bytes, uint32_t* win, int z, int nz) {
+    if (z + 2 < nz) store(win, z + 2);
+    if (z + 3 < nz) request(ref, plane_bytes, z + 3);
   }
 };
 
@@ -131,6 +174,9 @@ __global__ void __launch_bounds__(MarchGeo<S, TY>::NT, 1) split_march_kernel(con
   R* w_s = uxy_s + 6 * NM;                         // [3][5][NC]: u' (Guo: F), drho, 1/rho
   R* uz_s = w_s + 15 * NC;                         // [3][NC]
   FC* fc_s = reinterpret_cast<FC*>(uz_s + 3 * NC); // [DF][Q][NC]
+  uint32_t* fw_s = reinterpret_cast<uint32_t*>(fc_s + DF * Q * NC);   // [4][FW], local references only
+  uint32_t* gw_s = fw_s + 4 * GE::FW;                                 // [4][GW]
+  const size_t plane_bytes = (size_t)a.plane * sizeof(S);
 
   const int tile = (int)blockIdx.x;
   const int x0 = (tile % b.tiles_x) * 32, y0 = (tile / b.tiles_x) * TY;
@@ -155,14 +201,20 @@ __global__ void __launch_bounds__(MarchGeo<S, TY>::NT, 1) split_march_kernel(con
     }
     R inv1 = R(0), drho1 = R(0), jx1 = R(0), jy1 = R(0), jz1 = R(0);     // of the plane before
     MarchRaw<S> raw;
-    raw.request(b.fsrc, b.fref, a, ps, m);
+    raw.request(b.fsrc, a, ps, m);
+    RefFeed<GE::FWX, GE::FW, NM> feed;
+    if constexpr (IsLoc<S>::v) {
+      feed.set(a, t, x0 - 3, y0 - 3);
+      feed.start(b.fref, plane_bytes, fw_s, ps, nz);
+      bar_sync(BAR_M, NM);
+    }
     int uslot = 2;            // slot of plane p-1 in the rings of three
     for (int p = ps; p <= pe; ++p) {
       if (p >= ps + 2) bar_sync(BAR_D + (p & 1), NT);        // C of iteration p-2 is done
       R inv = R(0), drho = R(0), jx = R(0), jy = R(0), jz = R(0);
       if (p < nz) {
         R f[Q];
-        raw.decode(f);
+        raw.template decode<GE::FWX, GE::FW>(f, fw_s, (ry + 1) * GE::FWX + rx + 1, p, nz);
         if (COLLIDE && in_c) {
           FC* fc = fc_s + (size_t)(p & (DF - 1)) * Q * NC + ct;
 #pragma unroll
@@ -178,8 +230,9 @@ __global__ void __launch_bounds__(MarchGeo<S, TY>::NT, 1) split_march_kernel(con
         // behind the last use of f, so that its registers take the next request
         if (p + 1 < nz && p < pe) {
           m.advance(step);
-          raw.request(b.fsrc, b.fref, a, p + 1, m);
+          raw.request(b.fsrc, a, p + 1, m);
         }
+        if constexpr (IsLoc<S>::v) feed.next(b.fref, plane_bytes, fw_s, p, nz);
       }
       bar_sync(BAR_M, NM);
       const int q = p - 1;
@@ -232,7 +285,12 @@ __global__ void __launch_bounds__(MarchGeo<S, TY>::NT, 1) split_march_kernel(con
     }
     MarchRaw<S> raw;
     unsigned own = m.v[1][1];
-    raw.request(b.gsrc, b.gref, a, z0, m);
+    raw.request(b.gsrc, a, z0, m);
+    RefFeed<GE::GWX, GE::GW, NC> feed;
+    if constexpr (IsLoc<S>::v) {
+      feed.set(a, t, x0 - 1, y0 - 1);
+      feed.start(b.gref, plane_bytes, gw_s, z0, nz);     // the first ready barrier makes it visible
+    }
     R uzm = R(0), uz = R(0), uzp = R(0);
     int uslot = 2;            // slot of plane p-1 in the rings of three; plane p-2 has the one before
     for (int p = ps; p <= pe; ++p) {
@@ -252,7 +310,7 @@ __global__ void __launch_bounds__(MarchGeo<S, TY>::NT, 1) split_march_kernel(con
         const R* us = uxy_s + zslot * (2 * NM);
         const R* w = w_s + zslot * (5 * NC) + t;
         R g[Q];
-        raw.decode(g);
+        raw.template decode<GE::GWX, GE::GW>(g, gw_s, (ty + 1) * GE::GWX + tx + 1, z, nz);
         if (z == 0 || z == nz - 1)
           g_wall_fix<S, R>(g, static_cast<const S*>(a.fin), a.N, (int)(own / (unsigned)sizeof(S)), z, nz, kp.rho0, kp.T0,
                            kp.T_d, kp.T_u, kp.lam);
@@ -284,7 +342,7 @@ __global__ void __launch_bounds__(MarchGeo<S, TY>::NT, 1) split_march_kernel(con
                      [&](int l, R v) { putg(l, IsLoc<S>::v ? v - lrg[CSQ(l)] : v); });
           if (z + 1 < z1) {
             m.advance(step);
-            raw.request(b.gsrc, b.gref, a, z + 1, m);
+            raw.request(b.gsrc, a, z + 1, m);
           }
           const R wf[3] = {w[0], w[NC], w[2 * NC]};
           const FC* fc = fc_s + (size_t)(z & (DF - 1)) * Q * NC + t;
@@ -301,12 +359,15 @@ __global__ void __launch_bounds__(MarchGeo<S, TY>::NT, 1) split_march_kernel(con
           own += step;
           if (z + 1 < z1) {
             m.advance(step);
-            raw.request(b.gsrc, b.gref, a, z + 1, m);
+            raw.request(b.gsrc, a, z + 1, m);
           }
         }
       }
       if constexpr (DIAG) {
         if (a.part != nullptr && z >= z0) dt.template reduce<TY>(red[z & 1], ty, tx);
+      }
+      if constexpr (IsLoc<S>::v) {
+        if (z >= z0) feed.next(b.gref, plane_bytes, gw_s, z, nz);
       }
       if (p + 2 <= pe) bar_arrive(BAR_D + (p & 1), NT);
     }
