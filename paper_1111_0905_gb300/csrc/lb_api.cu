@@ -231,7 +231,7 @@ dim3 fused_grid(const lb_ctx* c) { return dim3(c->ntiles, c->nchunks); }
 
 cudaError_t launch_step(const lb_ctx* c, const KArgs& a, int mode) {
   if (c->form == lb_ctx::kThree) return c->ops->split(a, mode, c->three_nt, c->stream);
-  if (c->form == lb_ctx::kMarch) return c->ops->march(a, mode, c->march_zc, c->stream);
+  if (c->form == lb_ctx::kMarch) return c->ops->march(a, mode, c->march_zc, c->march_zc2, c->stream);
   return c->ops->fused(a, mode, c->by, fused_grid(c), c->stream);
 }
 
@@ -245,7 +245,8 @@ namespace {
 // FP32 compute takes the one-launch march, unless three kernels are expected to be faster. A march
 // iteration is one plane of a CTA; a CTA of zc planes takes zc + 4 of them and about two more to
 // start, one CTA per SM, in waves: ceil(CTAs / SMs) (zc + 6) iterations. Measured per iteration (128^3,
-// 256^3): FP32 1.8 us, 16-bit deviations 1.5 us, local references 2.2 us. The three kernels take about
+// 256^3): FP32 1.8 us, 16-bit deviations 1.5 us (two nodes per thread: 2.2 us for a tile of twice the
+// width, 7 rows), local references 2.2 us. The three kernels take about
 // 7 us and per node 73, 58 and 77 ps (FP32 64^3 28 us and 128^3 168 us, the march 21 and 126 us; 32^3
 // 7.6 us against 18; local references 96^3 72 us against 86). The chunk zc is the one of the least cost.
 cudaError_t choose_form(lb_ctx* c) {
@@ -257,18 +258,30 @@ cudaError_t choose_form(lb_ctx* c) {
   c->form = lb_ctx::kThree;
   if (c->ops->march_ty > 0) {
     const int nz = c->p.nz;
-    const long long tiles = (long long)c->tiles_x * ((c->p.ny + c->ops->march_ty - 1) / c->ops->march_ty);
-    long long best = -1;
-    for (int nch = 1; nch <= nz && nch <= 65535; ++nch) {
-      const int zc = (nz + nch - 1) / nch;
-      if (zc < 4 && nch > 1) break;
-      const long long ctas = tiles * ((nz + zc - 1) / zc);
-      const long long cost = ((ctas + sms - 1) / sms) * (zc + 6);
-      if (best < 0 || cost < best) { best = cost; c->march_zc = zc; }
-    }
+    // the least cost of a march over a number of tiles, and its chunk
+    auto chunk = [&](long long tiles, int* best_zc) {
+      long long best = -1;
+      for (int nch = 1; nch <= nz && nch <= 65535; ++nch) {
+        const int zc = (nz + nch - 1) / nch;
+        if (zc < 4 && nch > 1) break;
+        const long long ctas = tiles * ((nz + zc - 1) / zc);
+        const long long cost = ((ctas + sms - 1) / sms) * (zc + 6);
+        if (best < 0 || cost < best) { best = cost; *best_zc = zc; }
+      }
+      return best;
+    };
+    auto rows = [&](int ty) { return (long long)((c->p.ny + ty - 1) / ty); };
+    const long long tiles = (long long)c->tiles_x * rows(c->ops->march_ty);
+    const long long best = chunk(tiles, &c->march_zc);
     const bool b16 = c->ops->esize == 2, loc = c->ops->slots > Q;
-    const double iteration = loc ? 2.2e-6 : (b16 ? 1.5e-6 : 1.8e-6), node = loc ? 77e-12 : (b16 ? 58e-12 : 73e-12);
-    if (iteration * (double)best < 7e-6 + node * (double)c->N) {
+    const double node = loc ? 77e-12 : (b16 ? 58e-12 : 73e-12);
+    double march = (loc ? 2.2e-6 : (b16 ? 1.5e-6 : 1.8e-6)) * (double)best;
+    if (c->ops->march_ty2 > 0 && c->p.nx % 2 == 0) {
+      const double two = 2.2e-6 * (double)chunk((long long)((c->p.nx + 63) / 64) * rows(c->ops->march_ty2), &c->march_zc2);
+      if (two < march) march = two;
+      else c->march_zc2 = 0;
+    }
+    if (march < 7e-6 + node * (double)c->N) {
       c->form = lb_ctx::kMarch;
       c->nblk = (int)tiles;
       return cudaSuccess;

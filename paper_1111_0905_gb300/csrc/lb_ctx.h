@@ -29,7 +29,7 @@ struct lb_ctx {
   enum Form { kTile, kThree, kMarch } form = kTile;
   void* fld = nullptr;       // kThree: its fields, [8] (FP64: [12]) [N] in the compute precision
   int three_nt = 256;        // kThree: threads per CTA
-  int march_zc = 0;          // kMarch: planes per CTA
+  int march_zc = 0, march_zc2 = 0;   // kMarch: planes per CTA (one and two nodes per thread)
   int nblk = 0;              // CTAs per plane: diagnostics partials per plane
   long long step = 0;
   // the current state is due for a Nu sample (nu_every) that the next step's launch takes in

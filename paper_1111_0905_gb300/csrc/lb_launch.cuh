@@ -2,7 +2,7 @@
 // Each precision is compiled in its own translation unit (lb_prec_*.cu) that defines one table.
 #pragma once
 #include "lb_kernels.cuh"
-#include "lb_march.cuh"
+#include "lb_march2.cuh"
 
 namespace tlbm {
 
@@ -22,8 +22,9 @@ struct PrecOps {
   // the three-kernel step (lb_split.cuh) in mode MODE_* with CTAs of nt threads (64 or 256), and the
   // one-launch march (lb_march.cuh) with chunks of zc planes and its tile height (0: none for FP64)
   cudaError_t (*split)(const KArgs&, int mode, int nt, cudaStream_t);
-  cudaError_t (*march)(const KArgs&, int mode, int zc, cudaStream_t);
+  cudaError_t (*march)(const KArgs&, int mode, int zc, int zc2, cudaStream_t);
   int march_ty;
+  int march_ty2;       // tile height of the march with two nodes per thread (64 wide; chunks of zc2; 0: none)
   int slots;           // stored slots per lattice and node: 19, or 21 with the local references
 };
 
@@ -179,6 +180,13 @@ template <class S> struct OpsImpl {
   // 1.30, 1.34, 1.18, 1.42 ms. Taller tiles recompute fewer ring nodes but leave fewer registers per
   // thread, and a spilled value in flight makes its warp wait for it.
   static constexpr int MTY = IsLoc<S>::v ? 7 : 8;
+  // Two nodes per thread (lb_march2.cuh): 16-bit deviations, even nx, plain steps of the paper's scheme.
+  // Tile heights 5, 6, 7, 8 on the FP16 256^3 cell: 0.71, 0.67, 0.61, 0.76 ms (8 spills); the one-node
+  // march 0.72 ms.
+  static constexpr int MTY2 = sizeof(S) == 2 && !IsLoc<S>::v ? 7 : 0;
+  static bool pairs(const KArgs& a, int mode, int zc2) {
+    return MTY2 > 0 && zc2 > 0 && mode == MODE_STEP && (a.nx & 1) == 0 && variant_of(a.forcing, a.psi_kind) == 0;
+  }
   template <int VAR, int MODE> static cudaError_t march_go(const KArgs& a, const MarchArgs& b, dim3 grid, cudaStream_t st) {
     using GE = MarchGeo<S, MTY>;
     split_march_kernel<S, VAR, MODE, MTY><<<grid, GE::NT, GE::smem, st>>>(a, b);
@@ -193,6 +201,10 @@ template <class S> struct OpsImpl {
       return cudaSuccess;
     } else {
       cudaError_t e;
+      if constexpr (MTY2 > 0) {
+        if ((e = cudaFuncSetAttribute(split_march2_kernel<S, MTY2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)March2Geo<MTY2>::smem)) != cudaSuccess) return e;
+      }
       if ((e = march_attr<0, MODE_STEP>()) != cudaSuccess) return e;
       if ((e = march_attr<VAR_GUO, MODE_STEP>()) != cudaSuccess) return e;
       if ((e = march_attr<VAR_VDW, MODE_STEP>()) != cudaSuccess) return e;
@@ -202,7 +214,7 @@ template <class S> struct OpsImpl {
       return march_attr<VAR_VDW, MODE_MOMENTS>();
     }
   }
-  static cudaError_t march(const KArgs& a, int mode, int zc, cudaStream_t st) {
+  static cudaError_t march(const KArgs& a, int mode, int zc, int zc2, cudaStream_t st) {
     if constexpr (std::is_same<S, double>::value) {
       return cudaErrorInvalidValue;
     } else {
@@ -220,6 +232,16 @@ template <class S> struct OpsImpl {
       for (int k = 0; k < 2; ++k) {
         b.fref[k] = static_cast<const char*>(a.fin) + (Q + k) * N * es;
         b.gref[k] = static_cast<const char*>(a.gin) + (Q + k) * N * es;
+      }
+      if constexpr (MTY2 > 0) {
+        if (pairs(a, mode, zc2)) {
+          using GE = March2Geo<MTY2>;
+          b.tiles_x = (a.nx + GE::TX - 1) / GE::TX;
+          b.zc = zc2;
+          const dim3 grid((unsigned)(b.tiles_x * ((a.ny + MTY2 - 1) / MTY2)), (unsigned)((a.nz + zc2 - 1) / zc2));
+          split_march2_kernel<S, MTY2><<<grid, GE::NT, GE::smem, st>>>(a, b);
+          return cudaGetLastError();
+        }
       }
       b.tiles_x = (a.nx + BX - 1) / BX;
       b.zc = zc;

@@ -7,7 +7,7 @@ roundings of the compute precision. Tolerances, relative to the field's largest 
 of the parity tests: FP64 1e-12 and FP32 1e-5 on populations, rho, T and (with their floors) u; 16-bit
 2e-3 on populations, rho and T. No bound on u is asked of 16-bit storage: one rounding of a population
 of magnitude 2^-5 that falls the other way moves j by 2^-13 (BF16), more than 1e-2 of the floor. Sizes: one node past and short
-of a tile (32 x 8, 32 x 5), a warp and a chunk; one and two planes; the smallest cells that march."""
+of a tile (32 x 8, 32 x 7, 64 x 7), a warp and a chunk, one pair of nodes in a tile; one and two planes; the smallest cells that march."""
 import numpy as np
 import pytest
 import torch
@@ -72,13 +72,14 @@ def test_small_and_ragged_cells(lblib, cuda, prec, nx, ny, nz):
 
 
 # cells large enough to march (FP32 compute): exact tiles, one node past them, one short of them
-MARCH = [(96, 96, 96), (161, 105, 90), (127, 119, 77), (64, 200, 121)]
+MARCH = [(96, 96, 96), (161, 105, 90), (127, 119, 77), (64, 200, 121), (130, 99, 85), (192, 64, 128)]
 
 
 @pytest.mark.parametrize("prec", ["f32", "fp16loc", "fp16dev", "bf16dev"])
 @pytest.mark.parametrize("nx,ny,nz", MARCH)
-def test_march_cells(lblib, cuda, prec, nx, ny, nz):
-    p, rho, T = _cell(prec, nx, ny, nz, nu_every=1)
+@pytest.mark.parametrize("nu_every", [1, 0])     # steps that sample and plain steps are other kernels
+def test_march_cells(lblib, cuda, prec, nx, ny, nz, nu_every):
+    p, rho, T = _cell(prec, nx, ny, nz, nu_every=nu_every)
     _same(prec, p, rho, T, 3)
 
 
