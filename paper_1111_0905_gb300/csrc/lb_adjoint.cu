@@ -48,7 +48,7 @@ enum { AF_RHO = 0, AF_T, AF_UX, AF_UY, AF_UZ, AF_VX, AF_VY, AF_VZ, AF_D,
 // per-block parameter partials: wall terms of dJ/dT_d and dJ/dT_u, dJ/dG, the sum of J
 enum { P_TD = 0, P_TU, P_G, P_J, P_COUNT };
 
-constexpr int kThreads = 256;
+constexpr int kThreads = 128;     // coll_adj at 64^3: 124 us, 128 with 256
 
 // node of this thread: one CTA covers kThreads consecutive nodes of a plane
 struct Node {
@@ -78,8 +78,8 @@ __device__ __forceinline__ int at(const Geom& g, int x, int y, int z) {
 }
 
 // Sum of v over the CTA on thread 0, in a fixed order: every warp leaves its values in shared memory
-// and one adds them, 8 per lane and then by shuffles (12 FP64 instructions of one warp instead of 5
-// of every warp). sh is the caller's own array.
+// and one adds them, kThreads / 32 per lane and then by shuffles (8 FP64 instructions of one warp
+// instead of 5 of every warp). sh is the caller's own array.
 __device__ __forceinline__ double block_sum(double v, double* sh) {
   sh[threadIdx.x] = v;
   __syncthreads();
@@ -201,11 +201,13 @@ __device__ __forceinline__ AdjMoments adj_moments(const double (&a)[Q], const do
 // Wall rules^T, collision^T and the Nu terms. Bound by its FP64 instructions like everything here; the
 // moment form takes about 200 of them a node where the sum over the pairs took 650 (64^3: 128 us against
 // 288; the three reverse kernels 226 us against 388).
+// (The reverse kernels follow each other as the step's do: wait_for_predecessor in lb_split.cuh.)
 __global__ void __launch_bounds__(kThreads) coll_adj_kernel(const double* __restrict__ M, const double* __restrict__ Ln,
                                                             Geom g, Par p, double* __restrict__ A,
                                                             double* __restrict__ part) {
   __shared__ double sh[4][kThreads];
   const Node n = node_of(g);
+  wait_for_predecessor();
   const size_t N = (size_t)g.N, i = (size_t)n.z * (size_t)g.plane + n.i;
   const bool wallz = n.z == 0 || n.z == g.nz - 1;
   double pTd = 0.0, pTu = 0.0, pG = 0.0, pJ = 0.0;
@@ -299,6 +301,7 @@ __global__ void __launch_bounds__(kThreads) vel_adj_kernel(const double* __restr
                                                            double* __restrict__ A, double* __restrict__ part) {
   __shared__ double sh[kThreads];
   const Node n = node_of(g);
+  wait_for_predecessor();
   const size_t N = (size_t)g.N, plane = (size_t)g.plane, zo = (size_t)n.z * plane, i = zo + n.i;
   double pG = 0.0;
   if (n.valid) {
@@ -339,6 +342,7 @@ __global__ void __launch_bounds__(kThreads) vel_adj_kernel(const double* __restr
 __global__ void __launch_bounds__(kThreads) force_adj_kernel(const double* __restrict__ A, const double* __restrict__ Ln,
                                                              Geom g, Par p, double* __restrict__ L) {
   const Node n = node_of(g);
+  wait_for_predecessor();
   if (!n.valid) return;
   const size_t N = (size_t)g.N, plane = (size_t)g.plane, zo = (size_t)n.z * plane, i = zo + n.i;
   const double *Hx = A + AF_HX * N + zo, *Hy = A + AF_HY * N + zo, *Hz = A + AF_HZ * N + zo;
@@ -555,10 +559,10 @@ extern "C" int lb_adjoint_step(lb_ctx* c, long long nsteps, int checkpoint_every
       par.include_nu = (n >= 1) ? 1 : 0;
       double* Lcur = Lb[1 - li];
       const double* Lnext = have_next ? Lb[li] : nullptr;
-      coll_adj_kernel<<<(unsigned)parts, kThreads, 0, st>>>(Mn, Lnext, g, par, A, part);
-      vel_adj_kernel<<<(unsigned)parts, kThreads, 0, st>>>(Mn, g, par, A, part);
-      force_adj_kernel<<<(unsigned)parts, kThreads, 0, st>>>(A, Lnext, g, par, Lcur);
-      LB_CU(c, cudaGetLastError());
+      const unsigned pg = (unsigned)parts;
+      LB_CU(c, follow(coll_adj_kernel, pg, kThreads, st, Mn, Lnext, g, par, A, part));
+      LB_CU(c, follow(vel_adj_kernel, pg, kThreads, st, Mn, g, par, A, part));
+      LB_CU(c, follow(force_adj_kernel, pg, kThreads, st, static_cast<const double*>(A), Lnext, g, par, Lcur));
       li = 1 - li;
       have_next = true;
     }

@@ -194,7 +194,7 @@ KArgs make_args(const lb_ctx* c) {
         const double m = std::frexp(w2, &e);
         w2 = std::ldexp(std::nearbyint(std::ldexp(m, 20)), e - 20);
       }
-      om1 = (R)(1.0 - 36.0 * w2);
+      om1 = (R)(1.0 - (F32 ? 36.0 * w2 : omega));
       o[0] = (R)(12.0 * w2); o[1] = (R)(2.0 * w2); o[2] = (R)w2;
       for (int c = 0; c < 3; ++c) { s3[c] = (R)(3.0 * (double)o[c]); q[c] = (R)(4.5 * (double)o[c]); }
       return F32 ? 36.0 * w2 : omega;

@@ -6,6 +6,19 @@
 
 namespace tlbm {
 
+// Launch of a kernel that calls wait_for_predecessor first: it comes up as the CTAs of the launch before
+// it end (programmatic dependent launch).
+template <class... P, class... A>
+inline cudaError_t follow(void (*k)(P...), unsigned grid, int nt, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid); cfg.blockDim = dim3((unsigned)nt); cfg.stream = st;
+  cudaLaunchAttribute at = {};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at; cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k, args...);
+}
+
 struct PrecOps {
   size_t esize;        // bytes per stored population
   int deviation;       // 1 if populations are stored as deviations from w_l * ref
@@ -139,15 +152,6 @@ template <class S> struct OpsImpl {
   }
   // The three-kernel step (lb_split.cuh). NT threads per CTA: 256, or 64 for cells of few nodes per
   // SM, which smaller CTAs spread more evenly (FP64 32^3: see the rule in lb_api.cu).
-  template <class... P, class... A> static cudaError_t follow(void (*k)(P...), unsigned grid, int nt, cudaStream_t st, A... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid); cfg.blockDim = dim3((unsigned)nt); cfg.stream = st;
-    cudaLaunchAttribute at = {};
-    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &at; cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k, args...);
-  }
   template <int VAR, int NT> static cudaError_t three(const KArgs& a, int mode, cudaStream_t st) {
     const int nb = (a.plane + NT - 1) / NT;
     const unsigned grid = (unsigned)nb * (unsigned)a.nz;

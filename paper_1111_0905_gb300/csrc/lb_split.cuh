@@ -136,11 +136,12 @@ __device__ __forceinline__ float split_mv(float mi, const KPar<float>& kp) { ret
 
 // BGK relaxation of one lattice towards its equilibrium around the velocity v, pair by pair:
 //   out_l = om1 in_l + [ev + 9 (c.v)(c.F')] +- [s (c.v) + 3 (c.F')],  ev = q (c.v)^2 + P per class,
-// F' = 0 without Guo forcing. in(l) and put(l, value) access the populations.
-template <class R, bool GUO, class In, class Put>
+// F' = 0 without Guo forcing. in(l) and put(l, value) access the populations. FULL: om1 = 0 (relaxation
+// time 1), the populations themselves do not enter.
+template <class R, bool GUO, bool FULL = false, class In, class Put>
 __device__ __forceinline__ void relax(R om1, const R (&P)[3], const R (&q)[3], const R (&s)[3], R vx, R vy, R vz,
                                       const R (&F)[3], R ks, In in, Put put) {
-  put(0, fma_rn(om1, in(0), P[0]));
+  put(0, FULL ? P[0] : fma_rn(om1, in(0), P[0]));
 #pragma unroll
   for (int l = 1; l < Q; l += 2) {
     const R cv = cdot<R>(l, vx, vy, vz);
@@ -152,8 +153,8 @@ __device__ __forceinline__ void relax(R om1, const R (&P)[3], const R (&q)[3], c
       put(l, fma_rn(om1, in(l), ev) + od);
       put(OPP(l), fma_rn(om1, in(OPP(l)), ev) - od);
     } else {
-      put(l, fma_rn(s[CLS(l)], cv, fma_rn(om1, in(l), ev)));
-      put(OPP(l), fma_rn(-s[CLS(l)], cv, fma_rn(om1, in(OPP(l)), ev)));
+      put(l, fma_rn(s[CLS(l)], cv, FULL ? ev : fma_rn(om1, in(l), ev)));
+      put(OPP(l), fma_rn(-s[CLS(l)], cv, FULL ? ev : fma_rn(om1, in(OPP(l)), ev)));
     }
   }
 }
@@ -167,6 +168,13 @@ __device__ __forceinline__ void relax_g(const KPar<R>& kp, R E, R dE, R drho, R 
   const R P[3] = {kp.go[0] * (b0 - tg), kp.go[1] * b0, kp.go[2] * (b0 + tg)};
   const R q[3] = {R(0), kp.gq[1] * E, kp.gq[2] * E}, s[3] = {R(0), kp.gs[1] * E, kp.gs[2] * E};
   const R F[3] = {R(0), R(0), R(0)};
+  if constexpr (sizeof(R) == 8) {
+    // tau_kappa = 1: 18 of the 182 FP64 instructions of a collision less
+    if (kp.omk1 == R(0)) {
+      relax<R, false, true>(kp.omk1, P, q, s, ux, uy, uz, F, R(0), in, put);
+      return;
+    }
+  }
   relax<R, false>(kp.omk1, P, q, s, ux, uy, uz, F, R(0), in, put);
 }
 // f towards f^eq(rho, u', T) (w = u'), or with Guo forcing towards f^eq(rho, u, T) plus its source
