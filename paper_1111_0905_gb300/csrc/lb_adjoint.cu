@@ -199,8 +199,8 @@ __device__ __forceinline__ AdjMoments adj_moments(const double (&a)[Q], const do
 }
 
 // Wall rules^T, collision^T and the Nu terms. Bound by its FP64 instructions like everything here; the
-// moment form takes about 200 of them a node where the sum over the pairs took 650 (64^3: 128 us against
-// 288; the three reverse kernels 226 us against 388).
+// moment form takes about 200 of them a node where the sum over the pairs took 650 (64^3: 124 us against
+// 288; the three reverse kernels 222 us against 388).
 // (The reverse kernels follow each other as the step's do: wait_for_predecessor in lb_split.cuh.)
 __global__ void __launch_bounds__(kThreads) coll_adj_kernel(const double* __restrict__ M, const double* __restrict__ Ln,
                                                             Geom g, Par p, double* __restrict__ A,
@@ -296,7 +296,8 @@ __global__ void __launch_bounds__(kThreads) coll_adj_kernel(const double* __rest
 }
 
 // divergence^T (radius-1 gather), velocities^T: u = (j + F/2)/rho, u' = (j + tau F)/rho, the node's own
-// factors of force^T: F = -G psi A + rho g_z z, psi = e^{-1/rho}, and T = E/rho ^T
+// factors of force^T: F = -G psi A + rho g_z z, psi = e^{-1/rho}, and T = E/rho ^T. One reciprocal per
+// node serves this kernel and the next (64^3: 33 us).
 __global__ void __launch_bounds__(kThreads) vel_adj_kernel(const double* __restrict__ M, Geom g, Par p,
                                                            double* __restrict__ A, double* __restrict__ part) {
   __shared__ double sh[kThreads];
@@ -338,7 +339,8 @@ __global__ void __launch_bounds__(kThreads) vel_adj_kernel(const double* __restr
 
 // force^T's gather and moments^T. psi(y) enters F(x) for every link x + c_l = y: sum_l W_l c_l . H(y - c_l);
 // a ghost link of a wall plane (x + c_l beyond the wall, its mirror image y) is the same sum over the
-// plane's mirror image with H_z negated. Then lambda_l = (1 - om) lambda*_l + a_rho + c_l . a_j (g: + a_E).
+// plane's mirror image with H_z negated (33 FP64 additions; 18 dot products with their own loads took
+// 166 instructions). 64^3: 65 us against 80. Then lambda_l = (1 - om) lambda*_l + a_rho + c_l . a_j (g: + a_E).
 __global__ void __launch_bounds__(kThreads) force_adj_kernel(const double* __restrict__ A, const double* __restrict__ Ln,
                                                              Geom g, Par p, double* __restrict__ L) {
   const Node n = node_of(g);

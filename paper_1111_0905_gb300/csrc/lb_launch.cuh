@@ -32,7 +32,7 @@ struct PrecOps {
   cudaError_t (*info)(int by, int var, int out[4]);
   // store a given pre-collision state (float64 [19][N] f and g on the device) as the buffer
   cudaError_t (*setpops)(const KArgs&, const double*, const double*, cudaStream_t);
-  // the three-kernel step (lb_split.cuh) in mode MODE_* with CTAs of nt threads (64 or 256), and the
+  // the three-kernel step (lb_split.cuh) in mode MODE_* with CTAs of nt threads (32, 64 or 256), and the
   // one-launch march (lb_march.cuh) with chunks of zc planes and its tile height (0: none for FP64)
   cudaError_t (*split)(const KArgs&, int mode, int nt, cudaStream_t);
   cudaError_t (*march)(const KArgs&, int mode, int zc, int zc2, cudaStream_t);
@@ -150,8 +150,8 @@ template <class S> struct OpsImpl {
     if (by == 16) return go_by<16>(a, mode, grid, st);
     return cudaErrorInvalidValue;
   }
-  // The three-kernel step (lb_split.cuh). NT threads per CTA: 256, or 64 for cells of few nodes per
-  // SM, which smaller CTAs spread more evenly (FP64 32^3: see the rule in lb_api.cu).
+  // The three-kernel step (lb_split.cuh). NT threads per CTA: 256, or fewer for cells of few nodes per
+  // SM, which smaller CTAs spread more evenly (the rule stands in lb_api.cu).
   template <int VAR, int NT> static cudaError_t three(const KArgs& a, int mode, cudaStream_t st) {
     const int nb = (a.plane + NT - 1) / NT;
     const unsigned grid = (unsigned)nb * (unsigned)a.nz;
@@ -175,7 +175,7 @@ template <class S> struct OpsImpl {
     }
   }
   static cudaError_t split(const KArgs& a, int mode, int nt, cudaStream_t st) {
-    return nt == 64 ? three_var<64>(a, mode, st) : three_var<256>(a, mode, st);
+    return nt == 32 ? three_var<32>(a, mode, st) : (nt == 64 ? three_var<64>(a, mode, st) : three_var<256>(a, mode, st));
   }
 
   // The one-launch step (lb_march.cuh). Tile heights: measured on the 256^3 and 512^3 boiling cells,
