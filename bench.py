@@ -6,7 +6,7 @@ rho = 1.50 (1 + 0.01 xi) inside coexistence between a hot bottom and a cold top 
 Ra = half the largest value the adiabatic gradient allows at L = 512), FP32 form. The FP16- and
 BF16-deviation and FP64 forms of the same cell are timed beside it and stated with their error
 against the FP64 step. One "step" is one full time step of the method (pull streaming, moments,
-psi, force, velocities, divergence, f and g collisions, walls) = one fused kernel launch.
+psi, force, velocities, divergence, f and g collisions, walls): one launch at this size (FP64: three).
 Value = lattice-node updates per second (GLUPS) of the whole job.
 
   python bench.py [--gpus N --steps K --warmup W] [--impl reference]
@@ -42,30 +42,32 @@ STORED_SLOTS = {"f64": 19, "f32": 19, "bf16dev": 19, "fp16dev": 19, "fp16loc": 2
 # forms whose traffic is the 76 values per node of the yardstick lb_stream_bound (the FP64 form is
 # bound by its FP64 pipe; the local-reference form also loads the source nodes' references)
 PATTERN_FORMS = ("f32", "fp16dev", "bf16dev")
-KERNEL_TYPE = {"f64": "double", "f32": "float", "bf16dev": "__nv_bfloat16", "fp16dev": "__half",
-               "fp16loc": "tlbm::half_loc"}
+# the kernel that takes most of a step of the headline cell
+STEP_KERNEL = {"f64": "split_collide_kernel<double,0,0,256>", "f32": "split_march_kernel<float,0,0,8>",
+               "bf16dev": "split_march2_kernel<__nv_bfloat16,7>", "fp16dev": "split_march2_kernel<__half,7>",
+               "fp16loc": "split_march_kernel<tlbm::half_loc,0,0,7>"}
 
 # DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) per launch of the fused step
 # kernel from an ncu capture of a smaller cell (`nodes` nodes; a capture with more than the
 # launch time is kept to a few GB on the device), keyed by the hash of the kernel sources it
 # was taken on. The headline's traffic is that capture scaled by the node count (the traffic
 # of one launch grows in proportion to the nodes it updates); null once the sources changed.
-TRAFFIC = {"src_hash": "89f84465a4989b8a", "nodes": 192 ** 3,
-           "bytes_per_launch": {"f32": 1148334592 + 1032008960, "fp16loc": 602396672 + 553547520,
-                                "fp16dev": 543652608 + 495205632},
-           "what": "ncu DRAM bytes of one launch of the 192^3 paper-geometry cell, scaled by the node count"}
+TRAFFIC = {"src_hash": "a6c6f191f804461b", "nodes": 256 ** 3,
+           "bytes_per_launch": {"f32": 2659395584 + 2508636160, "fp16loc": 1455475456 + 1370433024,
+                                "fp16dev": 1294676224 + 1226098944},
+           "what": "ncu DRAM bytes of one launch of the 256^3 paper-geometry cell, scaled by the node count"}
 
-# FP64 operations per node of one FP64 step (ncu: 2 x DFMA + DADD + DMUL thread instructions of
-# one step of the 128^3 single-phase cell, i.e. the per-node pre-pass lb_fields_kernel,
-# 2 x 39,845,888 + 100,663,296, plus the step kernel, 2 x 327,282,688 + 91,111,424 + 129,517,568,
-# divided by its 2,097,152 nodes; the step kernel's count includes its chunk prologues, a smaller
-# share at 512^3), and GB300's nominal FP64 rate (152 SMs x 2 FP64 FMA per clock x 2 flops x 2.07
-# GHz = 1.26 TFLOP/s; no measured FP64 peak).
-FP64_FLOPS_PER_NODE = (2 * (39845888 + 327282688) + (100663296 + 91111424) + 129517568) / 2097152
+# FP64 operations per node of one FP64 step (ncu: 2 x DFMA + DADD + DMUL thread instructions of the
+# moments, velocity and collision kernels on the 128^3 boiling cell, divided by its 2,097,152 nodes),
+# and GB300's nominal FP64 rate (152 SMs x 2 FP64 FMA per clock x 2 flops x 2.07 GHz = 1.26 TFLOP/s; no
+# measured FP64 peak).
+FP64_FLOPS_PER_NODE = (2 * (39845888 + 23068672 + 214630400) + (88080384 + 37748736 + 86917120)
+                       + (12582912 + 82083840)) / 2097152
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
 
 
-STEP_KERNEL_SOURCES = ("lb_kernels.cuh", "lb_launch.cuh", "lb_prec_f32.cu", "lb_prec_f16.cu")
+STEP_KERNEL_SOURCES = ("lb_kernels.cuh", "lb_split.cuh", "lb_march.cuh", "lb_march2.cuh", "lb_launch.cuh",
+                       "lb_prec_f32.cu", "lb_prec_f16.cu")
 
 
 def kernel_src_hash() -> str:
@@ -399,7 +401,7 @@ def run_ours(args):
                 "frac": bytes_launch / (main["ms_per_step"] * 1e-3) / 1e9 / peaks["hbm_gbs"],
                 "traffic": traffic, "peak_src": peaks["src"] + " (MEASURED_PEAKS.json hbm_gbs, burst copy)",
                 "traffic_src": TRAFFIC["what"] if traffic is not None else "kernel sources changed since the capture",
-                "kernel": f"tlbm::lb_fused_kernel<{KERNEL_TYPE[main_form]},8,0,0>",
+                "kernel": f"tlbm::{STEP_KERNEL[main_form]}",
                 "algorithmic_bytes_per_launch": bytes_launch,
                 "algorithmic": f"76 values x {STORE_BYTES[main_form]} B x {N} nodes (19 f + 19 g read and written)"}
     pb = pattern.get(f"{STORE_BYTES[main_form]}B") if main_form in PATTERN_FORMS else None
@@ -409,7 +411,7 @@ def run_ours(args):
             "GBs": same["GBs"], "frac_of_peak": same["frac_of_peak"], "warps_per_sm": same["warps_per_sm"],
             "frac_achieved_of_it": roofline["achieved"] / same["GBs"],
             "what": "lb_stream_bound (the step's 76 loads and stores per node, no arithmetic) timed live "
-                    "at the fused kernel's resident warps per SM"}
+                    "at 16 resident warps per SM"}
 
     out = None
     if rank == 0:
@@ -431,9 +433,8 @@ def run_ours(args):
 
 
 def stream_bound_sweep(lb, torch, peaks, p, fused_ctas: int) -> dict:
-    """lb_stream_bound on the cell's grid in 4- and 2-byte elements: at the fused kernel's residency
-    (its CTAs per SM, 256 threads each like the fused kernel's), at the yardstick's own occupancy
-    limit, and one node per thread. 76 values per node per launch; inputs far larger than L2 and
+    """lb_stream_bound on the cell's grid in 4- and 2-byte elements: at the tile march's residency
+    (two CTAs of 256 threads per SM), at the yardstick's own occupancy limit, and one node per thread. 76 values per node per launch; inputs far larger than L2 and
     alternated between two pairs of lattices."""
     shape = (p.nz, p.ny, p.nx)
     N = p.nx * p.ny * p.nz
