@@ -155,14 +155,14 @@ __global__ void div_fwd_kernel(Geom g, double* __restrict__ M) {
 // lambda'_l(x + c_l), or through a wall the bounce-back that delivered f*_l(x) as f'_{opp(l)}(x) (g:
 // with a minus sign)
 template <bool G_LATTICE>
-__device__ __forceinline__ void adj_pull(double (&v)[Q], const double* __restrict__ Ln, const Geom& g, const Node& n) {
+__device__ __forceinline__ void adj_pull(double (&v)[Q], const double* Ln, const Geom& g, const Node& n) {
   const size_t N = (size_t)g.N, plane = (size_t)g.plane;
 #pragma unroll
   for (int l = 0; l < Q; ++l) {
     const int zn = n.z + CZ(l);
     const bool wall = zn < 0 || zn >= g.nz;
     const double* b = wall ? Ln + OPP(l) * N + (size_t)n.z * plane : Ln + l * N + (size_t)zn * plane;
-    const double x = __ldg(b + (wall ? n.i : n.xs[1 + CX(l)] + n.ys[1 + CY(l)]));
+    const double x = b[wall ? n.i : n.xs[1 + CX(l)] + n.ys[1 + CY(l)]];
     v[l] = G_LATTICE && wall ? -x : x;
   }
 }
@@ -201,10 +201,10 @@ __device__ __forceinline__ AdjMoments adj_moments(const double (&a)[Q], const do
 // Wall rules^T, collision^T and the Nu terms. Bound by its FP64 instructions like everything here; the
 // moment form takes about 200 of them a node where the sum over the pairs took 650 (64^3: 124 us against
 // 288; the three reverse kernels 222 us against 388).
-// (The reverse kernels follow each other as the step's do: wait_for_predecessor in lb_split.cuh.)
-__global__ void __launch_bounds__(kThreads) coll_adj_kernel(const double* __restrict__ M, const double* __restrict__ Ln,
-                                                            Geom g, Par p, double* __restrict__ A,
-                                                            double* __restrict__ part) {
+// (The reverse kernels follow each other as the step's do, and like them read through plain loads only:
+// wait_for_predecessor and ld_at in lb_split.cuh.)
+__global__ void __launch_bounds__(kThreads) coll_adj_kernel(const double* M, const double* Ln, Geom g, Par p,
+                                                            double* A, double* part) {
   __shared__ double sh[4][kThreads];
   const Node n = node_of(g);
   wait_for_predecessor();
@@ -298,8 +298,7 @@ __global__ void __launch_bounds__(kThreads) coll_adj_kernel(const double* __rest
 // divergence^T (radius-1 gather), velocities^T: u = (j + F/2)/rho, u' = (j + tau F)/rho, the node's own
 // factors of force^T: F = -G psi A + rho g_z z, psi = e^{-1/rho}, and T = E/rho ^T. One reciprocal per
 // node serves this kernel and the next (64^3: 33 us).
-__global__ void __launch_bounds__(kThreads) vel_adj_kernel(const double* __restrict__ M, Geom g, Par p,
-                                                           double* __restrict__ A, double* __restrict__ part) {
+__global__ void __launch_bounds__(kThreads) vel_adj_kernel(const double* M, Geom g, Par p, double* A, double* part) {
   __shared__ double sh[kThreads];
   const Node n = node_of(g);
   wait_for_predecessor();
@@ -313,24 +312,31 @@ __global__ void __launch_bounds__(kThreads) vel_adj_kernel(const double* __restr
                           aD[zo + n.xs[1] + n.ys[0]] - aD[zo + n.xs[1] + n.ys[2]], dm - dp};
     const double rho = M[MF_RHO * N + i], psi = M[MF_PSI * N + i];
     const double inv = 1.0 / rho;
+    double au[3], av[3], mu[3], mv[3], ma[3];       // every load before the first store
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      au[k] = A[(AF_UX + k) * N + i]; av[k] = A[(AF_VX + k) * N + i];
+      mu[k] = M[(MF_UX + k) * N + i]; mv[k] = M[(MF_VX + k) * N + i]; ma[k] = M[(MF_AX + k) * N + i];
+    }
+    const double aT = A[AF_T * N + i], ar = A[AF_RHO * N + i], T = M[MF_T * N + i];
     double dot = 0.0, FA = 0.0, lFz = 0.0;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-      const double lu = A[(AF_UX + k) * N + i] + 0.5 * gr[k], lv = A[(AF_VX + k) * N + i];
+      const double lu = au[k] + 0.5 * gr[k], lv = av[k];
       A[(AF_JX + k) * N + i] = (lv + lu) * inv;
       const double lF = (p.tau * lv + 0.5 * lu) * inv;
-      dot += M[(MF_VX + k) * N + i] * lv + M[(MF_UX + k) * N + i] * lu;
-      FA += lF * M[(MF_AX + k) * N + i];
+      dot += mv[k] * lv + mu[k] * lu;
+      FA += lF * ma[k];
       A[(AF_HX + k) * N + i] = psi * lF;
       if (k == 2) lFz = lF;
     }
-    const double aE = A[AF_T * N + i] * inv;
+    const double aE = aT * inv;
     const double kp = -p.G * psi * inv * inv;       // lambda_psi -> lambda_rho of the terms -G (...)
     pG = -psi * FA;
     A[AF_E * N + i] = aE;
     A[AF_KP * N + i] = kp * (1.0 / 12.0);
-    double a_rho = A[AF_RHO * N + i] - dot * inv + p.gz * lFz + kp * FA - aE * M[MF_T * N + i];
-    if (p.include_nu) a_rho += p.Kc * M[MF_UZ * N + i] * (0.5 * p.G * psi * psi) * inv;
+    double a_rho = ar - dot * inv + p.gz * lFz + kp * FA - aE * T;
+    if (p.include_nu) a_rho += p.Kc * mu[2] * (0.5 * p.G * psi * psi) * inv;
     A[AF_RHO * N + i] = a_rho;
   }
   const double s = block_sum(pG, sh);
@@ -341,8 +347,8 @@ __global__ void __launch_bounds__(kThreads) vel_adj_kernel(const double* __restr
 // a ghost link of a wall plane (x + c_l beyond the wall, its mirror image y) is the same sum over the
 // plane's mirror image with H_z negated (33 FP64 additions; 18 dot products with their own loads took
 // 166 instructions). 64^3: 65 us against 80. Then lambda_l = (1 - om) lambda*_l + a_rho + c_l . a_j (g: + a_E).
-__global__ void __launch_bounds__(kThreads) force_adj_kernel(const double* __restrict__ A, const double* __restrict__ Ln,
-                                                             Geom g, Par p, double* __restrict__ L) {
+__global__ void __launch_bounds__(kThreads) force_adj_kernel(const double* A, const double* Ln, Geom g, Par p,
+                                                             double* L) {
   const Node n = node_of(g);
   wait_for_predecessor();
   if (!n.valid) return;

@@ -280,6 +280,15 @@ __device__ __forceinline__ R wall_even_dev(int l, R drho_p, R rho0, R T0, R Tw, 
 template <class S>
 __device__ __forceinline__ float loc_ref(const S* __restrict__ buf, unsigned e, int ls, unsigned N);
 
+template <class R>
+__device__ __forceinline__ void g_wall_rule(R (&g)[Q], R dp, int z, int nz, R rho0, R T0, R Td, R Tu, R lam) {
+#pragma unroll
+  for (int l = 0; l < Q; ++l) {
+    if (CZ(l) > 0 && z == 0) g[l] = -g[l] + R(2) * wall_even_dev<R>(l, dp, rho0, T0, Td, lam);
+    if (CZ(l) < 0 && z == nz - 1) g[l] = -g[l] + R(2) * wall_even_dev<R>(l, dp, rho0, T0, Tu, lam);
+  }
+}
+
 template <class S, class R>
 __device__ __forceinline__ void g_wall_fix(R (&g)[Q], const S* __restrict__ fin, int N, int own,
                                            int z, int nz, R rho0, R T0, R Td, R Tu, R lam) {
@@ -297,11 +306,7 @@ __device__ __forceinline__ void g_wall_fix(R (&g)[Q], const S* __restrict__ fin,
 #pragma unroll
     for (int m = 1; m < Q; ++m) dp = dp + Store<S>::ld(fin + (size_t)m * N + own);
   }
-#pragma unroll
-  for (int l = 0; l < Q; ++l) {
-    if (CZ(l) > 0 && z == 0) g[l] = -g[l] + R(2) * wall_even_dev<R>(l, dp, rho0, T0, Td, lam);
-    if (CZ(l) < 0 && z == nz - 1) g[l] = -g[l] + R(2) * wall_even_dev<R>(l, dp, rho0, T0, Tu, lam);
-  }
+  g_wall_rule<R>(g, dp, z, nz, rho0, T0, Td, Tu, lam);
 }
 
 // MODE_STEP: one time step. MODE_MOMENTS: the moments of the current state (fields and/or the

@@ -36,14 +36,11 @@ __device__ __forceinline__ void neighbours(unsigned (&xs)[3], unsigned (&ys)[3],
   ys[0] = row == 0 ? last : row - nx; ys[1] = row; ys[2] = row == last ? 0u : row + nx;
 }
 
-// element i of a plane (the byte offset in a plane fits 32 bits)
+// Element i of a plane (the byte offset in a plane fits 32 bits). Plain loads: what a kernel reads here
+// the launch before it wrote, and it is up before those writes are complete (wait_for_predecessor), so
+// the read-only path, for memory that nobody writes while a kernel is up, is not for it.
 template <class T> __device__ __forceinline__ T ld_at(const T* base, unsigned i) {
-  return __ldg(reinterpret_cast<const T*>(reinterpret_cast<const char*>(base) + (size_t)(i * (unsigned)sizeof(T))));
-}
-template <> __device__ __forceinline__ half_loc ld_at<half_loc>(const half_loc* base, unsigned i) {
-  half_loc h;
-  h.h = __ldg(reinterpret_cast<const __half*>(reinterpret_cast<const char*>(base) + (size_t)(i * 2u)));
-  return h;
+  return *reinterpret_cast<const T*>(reinterpret_cast<const char*>(base) + (size_t)(i * (unsigned)sizeof(T)));
 }
 template <class T> __device__ __forceinline__ void st_at(T* base, unsigned i, T v) {
   *reinterpret_cast<T*>(reinterpret_cast<char*>(base) + (size_t)(i * (unsigned)sizeof(T))) = v;
@@ -65,7 +62,7 @@ __device__ __forceinline__ float recip(float x) {
 // The 19 populations pulled at a node of plane z of lattice buf (through a wall the bounce-back
 // source), with the local references added.
 template <class S, class R>
-__device__ __forceinline__ void split_pull(R (&v)[Q], const S* __restrict__ buf, size_t N, size_t plane, int nz,
+__device__ __forceinline__ void split_pull(R (&v)[Q], const S* buf, size_t N, size_t plane, int nz,
                                            int z, const unsigned (&xs)[3], const unsigned (&ys)[3]) {
   const unsigned own = xs[1] + ys[1];
   S raw[Q];
@@ -89,6 +86,22 @@ __device__ __forceinline__ void split_pull(R (&v)[Q], const S* __restrict__ buf,
       v[l] += cvt<S, R>(ld_at((CSQ(l) == 1 ? r1 : r2) + zs, through ? own : xs[1 - CX(l)] + ys[1 - CY(l)]));
     }
   }
+}
+
+// Density deviation of a wall node for the thermal wall rule: the sum of its own stored f (with their
+// local references), in the order of g_wall_fix.
+template <class S, class R>
+__device__ __forceinline__ R split_wall_density(const S* fin, size_t N, size_t o) {
+  auto at = [&](int l) -> R { return cvt<S, R>(ld_at(fin + l * N + o, 0u)); };
+  R ref[3] = {R(0), R(0), R(0)};
+  if constexpr (IsLoc<S>::v) {
+    ref[1] = at(Q); ref[2] = at(Q + 1);
+    ref[0] = R(12) * (ref[1] - ref[2]);
+  }
+  R dp = IsLoc<S>::v ? at(0) + ref[0] : at(0);
+#pragma unroll
+  for (int l = 1; l < Q; ++l) dp = dp + (IsLoc<S>::v ? at(l) + ref[CSQ(l)] : at(l));
+  return dp;
 }
 
 // Density and momentum deviations from the sums and differences of the opposite pairs (39 additions
@@ -316,6 +329,8 @@ __global__ void __launch_bounds__(NT) split_velocity_kernel(const KArgs a, int n
   pair_gradient<R>(d, A[0], A[1], A[2]);
   const KPar<R>& kp = kpar<R>(a);
   const R rv = ld_at(static_cast<const R*>(a.fd_rho) + zo, n.i);
+  const R j[3] = {ld_at(static_cast<const R*>(a.fd_j[0]) + zo, n.i), ld_at(static_cast<const R*>(a.fd_j[1]) + zo, n.i),
+                  ld_at(static_cast<const R*>(a.fd_j[2]) + zo, n.i)};
   const R rho = F64 ? rv : kp.rho0 + rv;
   R inv;
   if constexpr (F64) inv = ld_at(static_cast<const R*>(a.fd_inv) + zo, n.i);
@@ -325,8 +340,7 @@ __global__ void __launch_bounds__(NT) split_velocity_kernel(const KArgs a, int n
   const R mu = R(0.5) * mi, mv = split_mv(mi, kp);
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
-    const R j = ld_at(static_cast<const R*>(a.fd_j[k]) + zo, n.i);
-    const R ji = j * inv;
+    const R ji = j[k] * inv;
     st_at(static_cast<R*>(a.fd_u[k]) + zo, n.i, mu * A[k] + (k == 2 ? ji + kp.gz_u : ji));
     if constexpr (F64) {
       if constexpr (GUO) st_at(static_cast<R*>(a.fd_v[k]) + zo, n.i, k == 2 ? mg * A[k] + rho * kp.g_z : mg * A[k]);
@@ -386,7 +400,7 @@ __global__ void __launch_bounds__(NT, split_mb<S, MODE>() * 256 / NT) split_coll
     R inv;
     if constexpr (F64) inv = ld_at(static_cast<const R*>(a.fd_inv) + zo, o);
     if (z == 0 || z == a.nz - 1)
-      g_wall_fix<S, R>(g, fin, a.N, (int)(zo + o), z, a.nz, kp.rho0, kp.T0, kp.T_d, kp.T_u, kp.lam);
+      g_wall_rule<R>(g, split_wall_density<S, R>(fin, N, zo + o), z, a.nz, kp.rho0, kp.T0, kp.T_d, kp.T_u, kp.lam);
     const R rho = F64 ? rv : kp.rho0 + rv;
     const R drho = F64 ? rv - kp.rho0 : rv;
     if constexpr (!F64) inv = recip(rho);
@@ -420,8 +434,8 @@ __global__ void __launch_bounds__(NT, split_mb<S, MODE>() * 256 / NT) split_coll
           w[k] = GUO ? R(2) * (rho * u[k] - j[k]) : ji + split_mv(R(2) * (u[k] - ji), kp);   // u - j/rho = F/(2 rho)
         }
       }
-      S* __restrict__ fo = static_cast<S*>(a.fout) + zo;
-      S* __restrict__ go = static_cast<S*>(a.gout) + zo;
+      S* fo = static_cast<S*>(a.fout) + zo;
+      S* go = static_cast<S*>(a.gout) + zo;
       R lrf[3] = {R(0), R(0), R(0)}, lrg[3] = {R(0), R(0), R(0)};
       auto put = [&](S* base, int l, R v) {
         Store<S>::st(reinterpret_cast<S*>(reinterpret_cast<char*>(base + l * N) + (size_t)(o * (unsigned)sizeof(S))), v);
