@@ -39,6 +39,16 @@ template <class S, int TY> struct MarchGeo {
   // neighbourhood (radius 3 of the tile), of g on the tile's (radius 1)
   static constexpr int FWX = 38, FW = FWX * (TY + 6), GWX = 34, GW = GWX * (TY + 2);
   static constexpr size_t smem = 4 * floats + sizeof(FC) * DF * Q * NC + (IsLoc<S>::v ? 16 * (FW + GW) : 0);
+  // Ring node of thread t of the first group (the padding threads of its last warp repeat the last node;
+  // nobody reads what they form), and the node's word in a plane of f's window. A node reads the words
+  // of its eight neighbours in the planes below and above as well.
+  static __host__ __device__ constexpr int node(int t) { return t < NR ? t : NR - 1; }
+  static __host__ __device__ constexpr int fword(int t) { return (node(t) / RX + 1) * FWX + node(t) % RX + 1; }
+  static constexpr bool in_window() {
+    for (int t = 0; t < NM; ++t)
+      if (fword(t) - FWX - 1 < 0 || fword(t) + FWX + 1 >= FW) return false;
+    return true;
+  }
 };
 
 __device__ __forceinline__ void bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
@@ -196,7 +206,8 @@ __global__ void __launch_bounds__(MarchGeo<S, TY>::NT, 1) split_march_kernel(con
   const int ps = z0 >= 2 ? z0 - 2 : 0, pe = z1 + 1;
 
   if ((int)threadIdx.x < NM) {
-    const int t = (int)threadIdx.x, rx = t % RX, ry = t / RX;
+    static_assert(GE::in_window(), "a word outside the plane of the window belongs to another plane");
+    const int t = (int)threadIdx.x, rx = GE::node(t) % RX, ry = GE::node(t) / RX;
     const bool in_u = rx >= 1 && rx <= 34 && ry >= 1 && ry <= TY + 2;
     const bool in_c = rx >= 2 && rx <= 33 && ry >= 2 && ry <= TY + 1;
     const int ct = (ry - 2) * 32 + rx - 2;
@@ -221,7 +232,7 @@ __global__ void __launch_bounds__(MarchGeo<S, TY>::NT, 1) split_march_kernel(con
       R inv = R(0), drho = R(0), jx = R(0), jy = R(0), jz = R(0);
       if (p < nz) {
         R f[Q];
-        raw.template decode<GE::FWX, GE::FW>(f, fw_s, (ry + 1) * GE::FWX + rx + 1, p, nz);
+        raw.template decode<GE::FWX, GE::FW>(f, fw_s, GE::fword(t), p, nz);
         if (COLLIDE && in_c) {
           FC* fc = fc_s + (size_t)(p & (DF - 1)) * Q * NC + ct;
 #pragma unroll
