@@ -186,21 +186,20 @@ KArgs make_args(const lb_ctx* c) {
     constexpr bool F32 = sizeof(R) == 4;
     // x as R and, for FP32, its remainder
     auto two = [](double x, R& hi, R& lo) { hi = (R)x; lo = (R)(x - (double)hi); };
-    // the weights of relaxation rate omega; returns the rate that they add up to
-    auto weights = [](double omega, R& om1, R (&o)[3], R (&s3)[3], R (&q)[3]) -> double {
-      double w2 = omega / 36.0;
-      if (F32) {
-        int e;
-        const double m = std::frexp(w2, &e);
-        w2 = std::ldexp(std::nearbyint(std::ldexp(m, 20)), e - 20);
+    // the weights of relaxation rate omega; returns the rate that they and om1 add up to
+    auto weights = [&](double omega, R& om1, R (&o)[3], R (&o_lo)[3], R (&s3)[3], R (&s3_lo)[3], R (&q)[3]) -> double {
+      om1 = (R)(1.0 - omega);
+      const double rate = F32 ? 1.0 - (double)om1 : omega, w2 = rate / 36.0;
+      const double w[3] = {12.0 * w2, 2.0 * w2, w2};
+      for (int c = 0; c < 3; ++c) {
+        two(w[c], o[c], o_lo[c]);
+        two(3.0 * w[c], s3[c], s3_lo[c]);
+        q[c] = (R)(4.5 * w[c]);
       }
-      om1 = (R)(1.0 - (F32 ? 36.0 * w2 : omega));
-      o[0] = (R)(12.0 * w2); o[1] = (R)(2.0 * w2); o[2] = (R)w2;
-      for (int c = 0; c < 3; ++c) { s3[c] = (R)(3.0 * (double)o[c]); q[c] = (R)(4.5 * (double)o[c]); }
-      return F32 ? 36.0 * w2 : omega;
+      return rate;
     };
-    const double en = weights(a.omega_nu, k.om1, k.fo, k.fs, k.fq);
-    const double ek = weights(a.omega_kappa, k.omk1, k.go, k.gs, k.gq);
+    const double en = weights(a.omega_nu, k.om1, k.fo, k.fo_lo, k.fs, k.fs_lo, k.fq);
+    const double ek = weights(a.omega_kappa, k.omk1, k.go, k.go_lo, k.gs, k.gs_lo, k.gq);
     const double tau = F32 ? 1.0 / en : a.tau_nu;      // so that a step adds F to j, whole
     const bool dev = F32 && a.psi_kind != PSI_VDW;
     // the reference density of the FP32 forms is the rounded one (their deviations are from it)

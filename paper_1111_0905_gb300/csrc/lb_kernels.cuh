@@ -125,13 +125,14 @@ template <class R> struct KPar {
   R psi0, irho0;      // psi(rho0) = exp(-1/rho0) and 1/rho0 (deviation form of psi)
   // Constants of lb_split.cuh and lb_march.cuh. The force and the ideal pressure nearly cancel in the
   // flows of interest, so a relative rounding of 6e-8 in any one factor of either shows as a velocity
-  // error that is the same everywhere and adds up over the steps. In FP32 therefore the factors of F
-  // carry their rounding as a second float (_lo), and the weights per class (rest, axis, diagonal:
-  // w om, 3 w om, 4.5 w om) and 1 - om are exact multiples of one number (w om of a diagonal, rounded
-  // to 20 bits), so that mass, momentum and pressure relax consistently.
-  R om1, omk1, fo[3], fs[3], fq[3], go[3], gs[3], gq[3];
+  // error that is the same everywhere and adds up over the steps. In FP32 therefore the factors of F and
+  // the weights of the relaxation per class (rest, axis, diagonal: w om, 3 w om) carry their rounding as
+  // a second float (_lo), and om is 1 - om1 with om1 = 1 - 1/tau rounded: the rate that a context gets is
+  // within 3e-8 of its tau's (exact at tau = 1), and mass, momentum and pressure relax at that one rate.
+  // (fq = 4.5 w om, of the terms quadratic in the velocity, needs no second float.)
+  R om1, omk1, fo[3], fo_lo[3], fs[3], fs_lo[3], fq[3], go[3], go_lo[3], gs[3], gs_lo[3], gq[3];
   R mg, mg_lo;        // -G/12 (FP32, the paper's psi: -G psi(rho0)^2/12)
-  R irho0_lo, tau, tau_lo;   // tau = 1/(36 w om)
+  R irho0_lo, tau, tau_lo;   // tau = 1/om
   R gz_u, gz_v;       // g_z/2 and tau g_z
   R src, lam45;       // 1/(2 c_v omega_kappa), 4.5 lam
   R ks;               // 1 - omega_nu/2 (Guo forcing)

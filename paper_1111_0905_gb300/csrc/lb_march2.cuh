@@ -305,9 +305,11 @@ __global__ void __launch_bounds__(March2Geo<TY>::NT, 1) split_march2_kernel(cons
           const R uu = u[0][k] * u[0][k] + u[1][k] * u[1][k] + u[2][k] * u[2][k];
           const R b0 = e - E * (R(1.5) * uu + D2[k] * kp.src);
           const R tg = kp.lam45 * ((e - kp.T0 * drho[k]) * inv[k]) - R(1.5) * e;
-          A[k][0] = kp.go[0] * (b0 - tg); A[k][1] = kp.go[1] * b0; A[k][2] = kp.go[2] * (b0 + tg);
+          const R e3[3] = {b0 - tg, b0, b0 + tg};
 #pragma unroll
-          for (int c = 1; c < 3; ++c) { B[k][c] = kp.gq[c] * E; C[k][c] = kp.gs[c] * E; }
+          for (int c = 0; c < 3; ++c) A[k][c] = mul2(kp.go[c], kp.go_lo[c], e3[c]);
+#pragma unroll
+          for (int c = 1; c < 3; ++c) { B[k][c] = kp.gq[c] * E; C[k][c] = mul2(kp.gs[c], kp.gs_lo[c], E); }
         }
         if (wallz) out(b.gdst, kp.omk1, u, [&](int k, int l) { return gin(k, l, true); });
         else out(b.gdst, kp.omk1, u, [&](int k, int l) { return gin(k, l, false); });
@@ -323,9 +325,11 @@ __global__ void __launch_bounds__(March2Geo<TY>::NT, 1) split_march2_kernel(cons
           const R vv = v[0][k] * v[0][k] + v[1][k] * v[1][k] + v[2][k] * v[2][k];
           const R a0 = drho[k] - (R(1.5) * rho) * vv;
           const R th = R(4.5) * dE[k] - R(1.5) * drho[k];
-          A[k][0] = kp.fo[0] * (a0 - th); A[k][1] = kp.fo[1] * a0; A[k][2] = kp.fo[2] * (a0 + th);
+          const R e3[3] = {a0 - th, a0, a0 + th};
 #pragma unroll
-          for (int c = 1; c < 3; ++c) { B[k][c] = kp.fq[c] * rho; C[k][c] = kp.fs[c] * rho; }
+          for (int c = 0; c < 3; ++c) A[k][c] = mul2(kp.fo[c], kp.fo_lo[c], e3[c]);
+#pragma unroll
+          for (int c = 1; c < 3; ++c) { B[k][c] = kp.fq[c] * rho; C[k][c] = mul2(kp.fs[c], kp.fs_lo[c], rho); }
         }
         const uint32_t* fc = fc_s + (size_t)(z & (DF - 1)) * (Q * NN / 2) + ct / 2;
         out(b.fdst, kp.om1, v, [&](int k, int l) { return k == 0 ? P2::lo(fc[l * (NN / 2)]) : P2::hi(fc[l * (NN / 2)]); });

@@ -49,6 +49,10 @@ template <class T> __device__ __forceinline__ void st_at(T* base, unsigned i, T 
 __device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
 __device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 
+// c x of a constant c whose FP32 rounding is kept as a second float
+__device__ __forceinline__ double mul2(double c, double, double x) { return c * x; }
+__device__ __forceinline__ float mul2(float c, float lo, float x) { return fma_rn(c, x, lo * x); }
+
 // 1/x: the division for FP64; for FP32 Newton's iteration on the hardware approximation (its error
 // is squared, so the result is within one rounding of 1/x for normal x, and the correctly rounded
 // intrinsic's test for its slow path is saved)
@@ -143,12 +147,11 @@ __device__ __forceinline__ R split_mg(R psi, const KPar<R>& kp) {
   if constexpr (sizeof(R) == 8) return kp.mg * psi;
   else {
     const R p = VDW ? psi : R(1) + psi;
-    return fma_rn(kp.mg, p, kp.mg_lo * p);
+    return mul2(kp.mg, kp.mg_lo, p);
   }
 }
 // tau F-factor / rho from F-factor / rho
-__device__ __forceinline__ double split_mv(double mi, const KPar<double>& kp) { return kp.tau * mi; }
-__device__ __forceinline__ float split_mv(float mi, const KPar<float>& kp) { return fma_rn(kp.tau, mi, kp.tau_lo * mi); }
+template <class R> __device__ __forceinline__ R split_mv(R mi, const KPar<R>& kp) { return mul2(kp.tau, kp.tau_lo, mi); }
 
 // BGK relaxation of one lattice towards its equilibrium around the velocity v, pair by pair:
 //   out_l = om1 in_l + [ev + 9 (c.v)(c.F')] +- [s (c.v) + 3 (c.F')],  ev = q (c.v)^2 + P per class,
@@ -181,8 +184,9 @@ __device__ __forceinline__ void relax_g(const KPar<R>& kp, R E, R dE, R drho, R 
   const R uu = ux * ux + uy * uy + uz * uz;
   const R b0 = dE - E * (R(1.5) * uu + D2 * kp.src);
   const R tg = kp.lam45 * ((dE - kp.T0 * drho) * inv) - R(1.5) * dE;
-  const R P[3] = {kp.go[0] * (b0 - tg), kp.go[1] * b0, kp.go[2] * (b0 + tg)};
-  const R q[3] = {R(0), kp.gq[1] * E, kp.gq[2] * E}, s[3] = {R(0), kp.gs[1] * E, kp.gs[2] * E};
+  const R P[3] = {mul2(kp.go[0], kp.go_lo[0], b0 - tg), mul2(kp.go[1], kp.go_lo[1], b0), mul2(kp.go[2], kp.go_lo[2], b0 + tg)};
+  const R q[3] = {R(0), kp.gq[1] * E, kp.gq[2] * E};
+  const R s[3] = {R(0), mul2(kp.gs[1], kp.gs_lo[1], E), mul2(kp.gs[2], kp.gs_lo[2], E)};
   const R F[3] = {R(0), R(0), R(0)};
   if constexpr (sizeof(R) == 8) {
     // tau_kappa = 1: 18 of the 182 FP64 instructions of a collision less
@@ -201,8 +205,9 @@ __device__ __forceinline__ void relax_f(const KPar<R>& kp, R rho, R drho, R dE, 
   const R vv = vx * vx + vy * vy + vz * vz;
   const R a0 = drho - (R(1.5) * rho) * vv;
   const R th = R(4.5) * dE - R(1.5) * drho;
-  R P[3] = {kp.fo[0] * (a0 - th), kp.fo[1] * a0, kp.fo[2] * (a0 + th)};
-  const R q[3] = {R(0), kp.fq[1] * rho, kp.fq[2] * rho}, s[3] = {R(0), kp.fs[1] * rho, kp.fs[2] * rho};
+  R P[3] = {mul2(kp.fo[0], kp.fo_lo[0], a0 - th), mul2(kp.fo[1], kp.fo_lo[1], a0), mul2(kp.fo[2], kp.fo_lo[2], a0 + th)};
+  const R q[3] = {R(0), kp.fq[1] * rho, kp.fq[2] * rho};
+  const R s[3] = {R(0), mul2(kp.fs[1], kp.fs_lo[1], rho), mul2(kp.fs[2], kp.fs_lo[2], rho)};
   if constexpr (GUO) {
     // (1 - om/2) w_l [3 (c - u).F + 9 (c.u)(c.F)]: the part -3 u.F of the even terms
     const R uF = R(-3) * kp.ks * (ux * w[0] + uy * w[1] + uz * w[2]);
