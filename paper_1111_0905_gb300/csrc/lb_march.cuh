@@ -55,8 +55,8 @@ __device__ __forceinline__ void bar_sync(int id, int n) { asm volatile("bar.sync
 __device__ __forceinline__ void bar_arrive(int id, int n) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory"); }
 
 // Byte offsets of the nine (dx, dy) neighbours of a node, advanced plane by plane; with them a pull
-// is one 32-bit offset on a base that does not change over the march. (Element indices need fewer
-// instructions, one wide multiply-add per pull, but ran 10 % slower with FP16 storage.)
+// is one 32-bit offset on a base that does not change over the march. (With element indices instead FP16
+// storage ran 10 % slower.)
 template <class S> struct MarchPos {
   unsigned v[3][3];
   __device__ __forceinline__ void set(const unsigned (&xs)[3], const unsigned (&ys)[3], size_t zo) {
