@@ -202,9 +202,11 @@ KArgs make_args(const lb_ctx* c) {
     const double ek = weights(a.omega_kappa, k.omk1, k.go, k.go_lo, k.gs, k.gs_lo, k.gq);
     const double tau = F32 ? 1.0 / en : a.tau_nu;      // so that a step adds F to j, whole
     const bool dev = F32 && a.psi_kind != PSI_VDW;
-    // the reference density of the FP32 forms is the rounded one (their deviations are from it)
-    const double r0 = (double)k.rho0, p0 = std::exp(-1.0 / r0);
-    two(dev ? -a.G * p0 * p0 / 12.0 : -a.G / 12.0, k.mg, k.mg_lo);
+    // The reference density of the FP32 forms is the rounded one (their deviations are from it). psi refers
+    // to rho1, rho0 unless that is below 1/40: psi(rho1)^2 stays a normal float.
+    const double r0 = (double)k.rho0, r1 = std::max(r0, 1.0 / 40.0), p1 = std::exp(-1.0 / r1);
+    k.t1 = (R)(1.0 / r1 - 1.0 / r0);
+    two(dev ? -a.G * p1 * p1 / 12.0 : -a.G / 12.0, k.mg, k.mg_lo);
     R hi;
     two(1.0 / r0, hi, k.irho0_lo);
     k.irho0 = hi;

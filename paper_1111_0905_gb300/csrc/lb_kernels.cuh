@@ -131,11 +131,12 @@ template <class R> struct KPar {
   // within 3e-8 of its tau's (exact at tau = 1), and mass, momentum and pressure relax at that one rate.
   // (fq = 4.5 w om, of the terms quadratic in the velocity, needs no second float.)
   R om1, omk1, fo[3], fo_lo[3], fs[3], fs_lo[3], fq[3], go[3], go_lo[3], gs[3], gs_lo[3], gq[3];
-  R mg, mg_lo;        // -G/12 (FP32, the paper's psi: -G psi(rho0)^2/12)
+  R mg, mg_lo;        // -G/12 (FP32, the paper's psi: -G psi(rho1)^2/12)
   R irho0_lo, tau, tau_lo;   // tau = 1/om
   R gz_u, gz_v;       // g_z/2 and tau g_z
   R src, lam45;       // 1/(2 c_v omega_kappa), 4.5 lam
   R ks;               // 1 - omega_nu/2 (Guo forcing)
+  R t1;               // FP32, the paper's psi: 1/rho1 - 1/rho0, 0 unless rho0 is small
 };
 
 // Scheme variants (comparisons with the paper's scheme, which is variant 0 of each).

@@ -55,10 +55,11 @@ __device__ __forceinline__ float mul2(float c, float lo, float x) { return fma_r
 
 // 1/x: the division for FP64; for FP32 one step of Newton's iteration, r (2 - y r), on the hardware's
 // approximation r of 1/y (relative error at most 2^-23, which the step squares): within 0.501 of the
-// last place (every bit pattern is tested). y is x scaled by a power of two so that neither y nor 1/y is subnormal, over the whole
-// range of x, and 0 and the infinities keep the approximation's own result. It has no branch:
-// __frcp_rn in its place, the same results on the timed cells, made the FP16 256^3 cell 4.9 % slower
-// (two nodes per thread; this form 1.4 %, against a step that knows normal x only), local references 1.4 % (0.9).
+// last place (every bit pattern is tested). y is x scaled by a power of two, so that neither y nor 1/y
+// is subnormal over the whole range of x; 0 and the infinities keep the approximation's own result. No
+// branch: __frcp_rn in its place gave the same bits on the timed cells and made the FP16 256^3 cell
+// (two nodes per thread) 4.9 % slower, local references 1.4 %, FP32 0.8 %, all against a step that knew
+// normal x only; this form 1.4, 0.9 and 0.5 %.
 __device__ __forceinline__ double recip(double x) { return 1.0 / x; }
 __device__ __forceinline__ float recip(float x) {
   const float ax = fabsf(x);
@@ -136,19 +137,20 @@ __device__ __forceinline__ void pair_gradient(const R (&d)[Q / 2], R& ax, R& ay,
   az = R(2) * d[2] + ((d[5] - d[6]) + (d[7] - d[8]));
 }
 
-// psi of a node as the fields keep it. FP32 compute, the paper's psi: e = psi/psi(rho0) - 1 = e^t - 1,
-// t = 1/rho0 - 1/rho = drho/(rho rho0) (sum_l W_l c_l = 0, so the force sum may take e for psi; it then
-// adds small numbers).
+// psi of a node as the fields keep it. FP32 compute, the paper's psi: e = psi/psi(rho1) - 1 = e^t - 1,
+// t = 1/rho1 - 1/rho = drho/(rho rho0) + t1 (sum_l W_l c_l = 0, so the force sum may take e for psi; it
+// then adds small numbers). rho1 is the reference density or, where psi(rho0)^2 would leave the range of
+// floats, 1/40.
 template <class R, bool VDW>
 __device__ __forceinline__ R split_psi(R rho, R drho, R inv, const KPar<R>& kp) {
   if constexpr (VDW) return psi_vdw(rho, kp);
   else if constexpr (sizeof(R) == 8) return fexp(-inv);
   else {
     const R x = drho * inv;
-    return expm1_dev(fma_rn(x, kp.irho0, x * kp.irho0_lo));
+    return expm1_dev(fma_rn(x, kp.irho0, fma_rn(x, kp.irho0_lo, kp.t1)));
   }
 }
-// -G psi / 12 (FP32 compute, the paper's psi: times psi(rho0)) from psi as kept
+// -G psi / 12 (FP32 compute, the paper's psi: times psi(rho1)) from psi as kept
 template <class R, bool VDW>
 __device__ __forceinline__ R split_mg(R psi, const KPar<R>& kp) {
   if constexpr (sizeof(R) == 8) return kp.mg * psi;
