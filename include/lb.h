@@ -117,10 +117,10 @@ int lb_init(const lb_params* params, const double* rho_init, const double* T_ini
  * z_chunk) takes the tile march: per step one fused launch (FP64: after a pass that forms the moments
  * of every node). Otherwise the library chooses by precision and grid size between a march in one
  * launch with separate warps for the moments and the collision, and three streaming kernels
- * (moments, velocities, collision); the forms differ in rounding only. With 16-bit storage the steps
- * that take a Nu sample may run in another form than those between them, so nu_every can change the
- * populations by their rounding. A step pull-streams f and g (periodic x/y, bounce-back walls), takes
- * the moments of Eq. (8), the force of
+ * (moments, velocities, collision); the forms differ in rounding only. In the forms that it chooses a
+ * step that takes a Nu sample (nu_every) and one that does not leave the same populations, bit for bit,
+ * and so do runs with lb_nusselt, lb_diagnostics, lb_save or lb_load between their steps. A step
+ * pull-streams f and g (periodic x/y, bounce-back walls), takes the moments of Eq. (8), the force of
  * Eq. (9) with psi = exp(-1/rho) plus gravity rho g_z z (psi_kind selects the variant), the shifted
  * velocity u' = (j + tau_nu F)/rho (forcing selects the variant),
  * the physical velocity u = (j + F/2)/rho and its divergence, and collides f (temperature in

@@ -251,7 +251,7 @@ namespace {
 // 7 us and per node 73, 58 and 77 ps (FP32 64^3 28 us and 128^3 168 us, the march 21 and 126 us; 32^3
 // 7.6 us against 18; local references 96^3 72 us against 86). The chunk zc is the one of the least cost.
 cudaError_t choose_form(lb_ctx* c) {
-  c->nblk = c->ntiles;
+  c->nblk = c->nblk_step = c->ntiles;
   if (c->p.tile_y != 0 || c->p.z_chunk != 0) { c->form = lb_ctx::kTile; return cudaSuccess; }
   int sms = 0;
   const cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
@@ -277,14 +277,16 @@ cudaError_t choose_form(lb_ctx* c) {
     const bool b16 = c->ops->esize == 2, loc = c->ops->slots > Q;
     const double node = loc ? 77e-12 : (b16 ? 58e-12 : 73e-12);
     double march = (loc ? 2.2e-6 : (b16 ? 1.5e-6 : 1.8e-6)) * (double)best;
-    if (c->ops->march_ty2 > 0 && c->p.nx % 2 == 0) {
-      const double two = 2.2e-6 * (double)chunk((long long)((c->p.nx + 63) / 64) * rows(c->ops->march_ty2), &c->march_zc2);
+    const long long tiles2 = c->ops->march_ty2 > 0 ? (long long)((c->p.nx + 63) / 64) * rows(c->ops->march_ty2) : 0;
+    if (tiles2 > 0 && c->p.nx % 2 == 0 && variant_of(c->p.forcing, c->p.psi_kind) == 0) {
+      const double two = 2.2e-6 * (double)chunk(tiles2, &c->march_zc2);
       if (two < march) march = two;
       else c->march_zc2 = 0;
     }
     if (march < 7e-6 + node * (double)c->N) {
       c->form = lb_ctx::kMarch;
       c->nblk = (int)tiles;
+      c->nblk_step = c->march_zc2 > 0 ? (int)tiles2 : c->nblk;
       return cudaSuccess;
     }
   }
@@ -296,7 +298,7 @@ cudaError_t choose_form(lb_ctx* c) {
     auto fullest = [&](int nt) { return ((long long)((c->plane + nt - 1) / nt) * c->p.nz + sms - 1) / sms * nt; };
     c->three_nt = fullest(64) > 64 && fullest(32) < fullest(64) ? 32 : 64;
   }
-  c->nblk = (c->plane + c->three_nt - 1) / c->three_nt;
+  c->nblk = c->nblk_step = (c->plane + c->three_nt - 1) / c->three_nt;
   return cudaSuccess;
 }
 
@@ -311,8 +313,8 @@ void free_all(lb_ctx* c) {
 
 // Moments pass into the plane partials, then Nu(z) and the global health values into diag;
 // Nu_mean is added to acc[0] (and 1 to acc[1]) when acc is not null.
-int finalize_diag(lb_ctx* c, double* acc) {
-  lb_diag_planes<<<c->p.nz, 128, 0, c->stream>>>(c->part, c->p.nz, c->nblk, c->diag);
+int finalize_diag(lb_ctx* c, double* acc, int nblk) {
+  lb_diag_planes<<<c->p.nz, 128, 0, c->stream>>>(c->part, c->p.nz, nblk, c->diag);
   const int ft = std::min(1024, (c->p.nz + 31) / 32 * 32);
   lb_diag_finalize<<<1, ft, 0, c->stream>>>(c->p.nz, c->p.nx * c->p.ny, c->p.kappa, c->p.T_d,
                                                c->p.T_u, c->diag, acc);
@@ -324,7 +326,7 @@ int run_diag_acc(lb_ctx* c, double* acc) {
   KArgs a = make_args(c);
   a.part = c->part;
   LB_CU(c, launch_step(c, a, MODE_MOMENTS));
-  return finalize_diag(c, acc);
+  return finalize_diag(c, acc, c->nblk);
 }
 
 int run_diag(lb_ctx* c, bool accumulate) { return run_diag_acc(c, accumulate ? c->nu_acc : nullptr); }
@@ -507,7 +509,7 @@ int lb_init(const lb_params* params, const double* rho_init, const double* T_ini
     cudaFree(staging);
     return bail(LB_ENOMEM);
   }
-  if (cudaMalloc(&c->part, (size_t)p.nz * c->nblk * NPART * sizeof(double)) != cudaSuccess ||
+  if (cudaMalloc(&c->part, (size_t)p.nz * std::max(c->nblk, c->nblk_step) * NPART * sizeof(double)) != cudaSuccess ||
       cudaMalloc(&c->diag, (size_t)(8 * p.nz + 8) * sizeof(double)) != cudaSuccess ||
       cudaMalloc(&c->nu_acc, 2 * sizeof(double)) != cudaSuccess) {
     cudaFree(staging);
@@ -539,7 +541,7 @@ int lb_step(lb_ctx* c, long long nsteps) {
       a.part = c->part;
       LB_CU(c, launch_step(c, a, MODE_STEP_DIAG));
       c->sample_pending = false;
-      const int rc = finalize_diag(c, c->nu_acc);
+      const int rc = finalize_diag(c, c->nu_acc, c->nblk_step);
       if (rc) return rc;
     } else {
       const int rc = flush_sample(c);

@@ -18,7 +18,7 @@ struct lb_ctx {
   int N = 0, plane = 0;
   int by = 8, zc = 0, tiles_x = 0, tiles_y = 0, ntiles = 0, nchunks = 0;
   double lam = 0.0, rho0 = 0.0, T0 = 0.0;
-  double* part = nullptr;    // [nz][ntiles][NPART]
+  double* part = nullptr;    // [nz][nblk or nblk_step][NPART]
   double* diag = nullptr;    // [nz + 8]
   double* nu_acc = nullptr;  // [2]
   double* fields = nullptr;  // [5][N] staging for host-bound lb_moments
@@ -30,7 +30,8 @@ struct lb_ctx {
   void* fld = nullptr;       // kThree: its fields, [8] (FP64: [12]) [N] in the compute precision
   int three_nt = 256;        // kThree: threads per CTA
   int march_zc = 0, march_zc2 = 0;   // kMarch: planes per CTA (one and two nodes per thread)
-  int nblk = 0;              // CTAs per plane: diagnostics partials per plane
+  // CTAs per plane, the diagnostics partials of a plane: of a moments pass, and of a step that samples
+  int nblk = 0, nblk_step = 0;
   long long step = 0;
   // the current state is due for a Nu sample (nu_every) that the next step's launch takes in
   // passing (fused step + diagnostics); lb_nusselt, lb_diagnostics, lb_save and
@@ -61,5 +62,5 @@ dim3 fused_grid(const lb_ctx* c);
 cudaError_t launch_step(const lb_ctx* c, const tlbm::KArgs& a, int mode);  // MODE_* over the whole cell
 int run_diag(lb_ctx* c, bool accumulate);
 int run_diag_acc(lb_ctx* c, double* acc);
-int finalize_diag(lb_ctx* c, double* acc);   // Nu(z) and health values from the partials
+int finalize_diag(lb_ctx* c, double* acc, int nblk);   // Nu(z) and health values from nblk partials a plane
 int flush_sample(lb_ctx* c);                 // take a pending Nu sample (moments pass)

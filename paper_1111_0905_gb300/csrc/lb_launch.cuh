@@ -184,12 +184,13 @@ template <class S> struct OpsImpl {
   // 1.30, 1.34, 1.18, 1.42 ms. Taller tiles recompute fewer ring nodes but leave fewer registers per
   // thread, and a spilled value in flight makes its warp wait for it.
   static constexpr int MTY = IsLoc<S>::v ? 7 : 8;
-  // Two nodes per thread (lb_march2.cuh): 16-bit deviations, even nx, plain steps of the paper's scheme.
+  // Two nodes per thread (lb_march2.cuh): 16-bit deviations, even nx, steps of the paper's scheme, sampling
+  // or not: one form for all steps of a context, so that a sample does not change them.
   // Tile heights 5, 6, 7, 8 on the FP16 256^3 cell: 0.71, 0.67, 0.61, 0.76 ms (8 spills); the one-node
   // march 0.72 ms.
   static constexpr int MTY2 = sizeof(S) == 2 && !IsLoc<S>::v ? 7 : 0;
   static bool pairs(const KArgs& a, int mode, int zc2) {
-    return MTY2 > 0 && zc2 > 0 && mode == MODE_STEP && (a.nx & 1) == 0 && variant_of(a.forcing, a.psi_kind) == 0;
+    return MTY2 > 0 && zc2 > 0 && mode != MODE_MOMENTS && (a.nx & 1) == 0 && variant_of(a.forcing, a.psi_kind) == 0;
   }
   template <int VAR, int MODE> static cudaError_t march_go(const KArgs& a, const MarchArgs& b, dim3 grid, cudaStream_t st) {
     using GE = MarchGeo<S, MTY>;
@@ -206,8 +207,11 @@ template <class S> struct OpsImpl {
     } else {
       cudaError_t e;
       if constexpr (MTY2 > 0) {
-        if ((e = cudaFuncSetAttribute(split_march2_kernel<S, MTY2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)March2Geo<MTY2>::smem)) != cudaSuccess) return e;
+        const int smem2 = (int)March2Geo<MTY2>::smem;
+        if ((e = cudaFuncSetAttribute(split_march2_kernel<S, MTY2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      smem2)) != cudaSuccess) return e;
+        if ((e = cudaFuncSetAttribute(split_march2_kernel<S, MTY2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      smem2)) != cudaSuccess) return e;
       }
       if ((e = march_attr<0, MODE_STEP>()) != cudaSuccess) return e;
       if ((e = march_attr<VAR_GUO, MODE_STEP>()) != cudaSuccess) return e;
@@ -243,7 +247,8 @@ template <class S> struct OpsImpl {
           b.tiles_x = (a.nx + GE::TX - 1) / GE::TX;
           b.zc = zc2;
           const dim3 grid((unsigned)(b.tiles_x * ((a.ny + MTY2 - 1) / MTY2)), (unsigned)((a.nz + zc2 - 1) / zc2));
-          split_march2_kernel<S, MTY2><<<grid, GE::NT, GE::smem, st>>>(a, b);
+          if (mode == MODE_STEP) split_march2_kernel<S, MTY2, false><<<grid, GE::NT, GE::smem, st>>>(a, b);
+          else split_march2_kernel<S, MTY2, true><<<grid, GE::NT, GE::smem, st>>>(a, b);
           return cudaGetLastError();
         }
       }

@@ -4,8 +4,8 @@
 // half of them addresses, conversions and stores that a pair of neighbours can share: populations
 // without an x shift are pulled, kept and stored as 4-byte words, psi and the velocities are read and
 // written in pairs, and a 64-wide tile recomputes fewer ring nodes. For even nx (a pair never crosses
-// the periodic edge and every word is aligned), the paper's scheme, plain steps; everything else takes
-// the one-node march. 832 instructions a node; FP16 256^3 boiling cell 722 -> 605 us a step, 512^3
+// the periodic edge and every word is aligned) and the paper's scheme; everything else takes the one-node
+// march. 832 instructions a node; FP16 256^3 boiling cell 722 -> 605 us a step, 512^3
 // 5.58 -> 4.82 ms, 128^3 105 -> 84 us.
 #pragma once
 #include "lb_march.cuh"
@@ -99,13 +99,16 @@ __device__ __forceinline__ void pair_advance(unsigned (&v)[3][3], unsigned bytes
     for (int dy = 0; dy < 3; ++dy) v[dx][dy] += bytes;
 }
 
-template <class S, int TY>
+// DIAG: a step that also forms the diagnostics partials of the state it reads. The step itself is the same
+// operation for operation, so a sample leaves the populations as they are without it. FP16 256^3: 657 us
+// with its finalisation, 612 without a sample (1219 when sampling steps took the one-node march).
+template <class S, int TY, bool DIAG>
 __global__ void __launch_bounds__(March2Geo<TY>::NT, 1) split_march2_kernel(const KArgs a, const MarchArgs b) {
   using R = float;
   using GE = March2Geo<TY>;
   using P2 = Pair16<S>;
   constexpr int NM = GE::NM, NT = GE::NT, NR = GE::NR, NN = GE::NN, RX = GE::RX, DF = GE::DF;
-  constexpr int BAR_M = 1, BAR_R = 2, BAR_D = 4;      // as in split_march_kernel
+  constexpr int BAR_M = 1, BAR_R = 2, BAR_D = 4, BAR_C = 6;      // as in split_march_kernel
   extern __shared__ __align__(16) unsigned char smem_raw[];
   R* psi_s = reinterpret_cast<R*>(smem_raw);       // [4][NR], two floats before the first row of a plane
   R* st_s = psi_s + 4 * NR;                        // [2][5][2 NM]: drho, j, 1/rho, by thread
@@ -217,6 +220,7 @@ __global__ void __launch_bounds__(March2Geo<TY>::NT, 1) split_march2_kernel(cons
       uslot = uslot == 2 ? 0 : uslot + 1;
     }
   } else {
+    __shared__ R red[DIAG ? 2 : 1][7][DIAG ? TY : 1];
     const int t = (int)threadIdx.x - NM, px = t & 31, ty = t >> 5;
     const int x = x0 + 2 * px, y = y0 + ty;
     const bool valid = x < a.nx && y < a.ny;
@@ -231,6 +235,12 @@ __global__ void __launch_bounds__(March2Geo<TY>::NT, 1) split_march2_kernel(cons
     for (int p = ps; p <= pe; ++p) {
       bar_sync(BAR_R + (p & 1), NT);
       const int z = p - 2;
+      if constexpr (DIAG) {
+        // the partials of the plane before are complete
+        if (z - 1 >= z0 && ty == 0)
+          diag_combine<R, TY>(red[(z - 1) & 1], px, a.part + ((size_t)(z - 1) * gridDim.x + blockIdx.x) * NPART);
+      }
+      DiagTerms<R> dt[2];
       uzm = uz; uz = uzp;
       if (p >= 1 && p - 1 < nz) uzp = ld2(uz_s + uslot * NN + ct);
       const int zslot = uslot == 0 ? 2 : uslot - 1;
@@ -302,6 +312,8 @@ __global__ void __launch_bounds__(March2Geo<TY>::NT, 1) split_march2_kernel(cons
           }
           dE[k] = e;
           const R E = kp.E0 + e;
+          if constexpr (DIAG)
+            dt[k].template take<false>(a, kp.rho0 + drho[k], inv[k], E * inv[k], E, u[0][k], u[1][k], u[2][k]);
           const R uu = u[0][k] * u[0][k] + u[1][k] * u[1][k] + u[2][k] * u[2][k];
           const R b0 = e - E * (R(1.5) * uu + D2[k] * kp.src);
           const R tg = kp.lam45 * ((e - kp.T0 * drho[k]) * inv[k]) - R(1.5) * e;
@@ -335,7 +347,17 @@ __global__ void __launch_bounds__(March2Geo<TY>::NT, 1) split_march2_kernel(cons
         out(b.fdst, kp.om1, v, [&](int k, int l) { return k == 0 ? P2::lo(fc[l * (NN / 2)]) : P2::hi(fc[l * (NN / 2)]); });
         own += step;
       }
+      if constexpr (DIAG) {
+        if (z >= z0) {
+          dt[0].add(dt[1]);
+          dt[0].template reduce<TY, true>(red[z & 1], ty, px);
+        }
+      }
       if (p + 2 <= pe) bar_arrive(BAR_D + (p & 1), NT);
+    }
+    if constexpr (DIAG) {
+      bar_sync(BAR_C, GE::NC);
+      if (ty == 0) diag_combine<R, TY>(red[(z1 - 1) & 1], px, a.part + ((size_t)(z1 - 1) * gridDim.x + blockIdx.x) * NPART);
     }
   }
 }

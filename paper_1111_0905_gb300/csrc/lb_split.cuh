@@ -229,7 +229,7 @@ __device__ __forceinline__ void relax_f(const KPar<R>& kp, R rho, R drho, R dE, 
 // U = c_v T + int_0^rho P_NI/s^2 ds: (G/4) e^{-2/rho}, or -T_v ln(1 - b rho) - a rho (vdW).
 template <class R> struct DiagTerms {
   R conv = R(0), T = R(0), rho = R(0), E = R(0), mr = R(sizeof(R) == 8 ? 1e300 : 3.0e38), mT = mr;
-  bool bad = false;
+  bool bad = false, bad2 = false;
   template <bool VDW>
   __device__ __forceinline__ void take(const KArgs& a, R r, R inv, R t, R e, R ux, R uy, R uz) {
     const KPar<R>& kp = kpar<R>(a);
@@ -242,9 +242,15 @@ template <class R> struct DiagTerms {
     T = t; rho = r; E = e; mr = r; mT = t;
     bad = !(isfinite(r) && isfinite(t) && isfinite(ux) && isfinite(uy) && isfinite(uz));
   }
+  // a second node's terms as well (reduce with PAIR)
+  __device__ __forceinline__ void add(const DiagTerms& b) {
+    conv += b.conv; T += b.T; rho += b.rho; E += b.E;
+    mr = fmin(mr, b.mr); mT = fmin(mT, b.mT);
+    bad2 = b.bad;
+  }
   // Warp sums in the compute precision into red[7][NW] (column w). The four sums are reduced together,
   // each exchange halving the values a lane carries (6 shuffles instead of 20), the two minima likewise.
-  template <int NW> __device__ __forceinline__ void reduce(R (&red)[7][NW], int w, int lane) {
+  template <int NW, bool PAIR = false> __device__ __forceinline__ void reduce(R (&red)[7][NW], int w, int lane) {
     const bool hi = (lane & 16) != 0, mid = (lane & 8) != 0;
     const R p = (hi ? rho : conv) + __shfl_xor_sync(0xffffffffu, hi ? conv : rho, 16);
     const R q = (hi ? E : T) + __shfl_xor_sync(0xffffffffu, hi ? T : E, 16);
@@ -256,7 +262,8 @@ template <class R> struct DiagTerms {
       s += __shfl_xor_sync(0xffffffffu, s, o);
       m = fmin(m, __shfl_xor_sync(0xffffffffu, m, o));
     }
-    const int nbad = __popc(__ballot_sync(0xffffffffu, bad));
+    int nbad = __popc(__ballot_sync(0xffffffffu, bad));
+    if constexpr (PAIR) nbad += __popc(__ballot_sync(0xffffffffu, bad2));
     // lanes 0, 8, 16, 24 hold conv, T, rho, E; lanes 0 and 16 the minima
     if ((lane & 7) == 0) red[lane >> 3][w] = s;
     if ((lane & 15) == 0) red[4 + (lane >> 4)][w] = m;
