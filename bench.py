@@ -273,7 +273,7 @@ def run_ours(args):
         if args.only:
             p.nu_every = args.nu_every
         lat = lb.Lattice(p, rho_d, T_d)
-        launch = lat.launch_info()
+        launch = lat.step_info()
         K = args.steps if (form == main_form or form != "f64") else min(args.steps, F64_MAX_STEPS)
         sampler = ClockSampler(uuid) if form == main_form else None
         ms = time_steps(lat, K, args.warmup, sampler)
@@ -297,7 +297,7 @@ def run_ours(args):
         torch.cuda.empty_cache()
 
     # the bound of the access pattern itself: the step's loads and stores without its arithmetic
-    pattern = stream_bound_sweep(lb, torch, peaks, p0, results[main_form]["launch"]["ctas_per_sm"])
+    pattern = stream_bound_sweep(lb, torch, peaks, p0, results[main_form]["launch"])
     for form in results:
         b = pattern.get(f"{STORE_BYTES[form]}B") if form in PATTERN_FORMS else None
         if b is not None:
@@ -411,7 +411,7 @@ def run_ours(args):
             "GBs": same["GBs"], "frac_of_peak": same["frac_of_peak"], "warps_per_sm": same["warps_per_sm"],
             "frac_achieved_of_it": roofline["achieved"] / same["GBs"],
             "what": "lb_stream_bound (the step's 76 loads and stores per node, no arithmetic) timed live "
-                    "at 16 resident warps per SM"}
+                    "at the resident warps per SM nearest to the step kernel's"}
 
     out = None
     if rank == 0:
@@ -432,10 +432,12 @@ def run_ours(args):
     return out
 
 
-def stream_bound_sweep(lb, torch, peaks, p, fused_ctas: int) -> dict:
-    """lb_stream_bound on the cell's grid in 4- and 2-byte elements: at the tile march's residency
-    (two CTAs of 256 threads per SM), at the yardstick's own occupancy limit, and one node per thread. 76 values per node per launch; inputs far larger than L2 and
-    alternated between two pairs of lattices."""
+def stream_bound_sweep(lb, torch, peaks, p, step: dict) -> dict:
+    """lb_stream_bound on the cell's grid in 4- and 2-byte elements: at the residency nearest to that of the
+    step's kernel (`step`, lb_step_info) in CTAs of 256 threads, at the yardstick's own occupancy limit,
+    and one node per thread. 76 values per node per launch; inputs far larger than L2 and alternated
+    between two pairs of lattices."""
+    fused_ctas = max(1, round(step["ctas_per_sm"] * step["threads_per_cta"] / 256))
     shape = (p.nz, p.ny, p.nx)
     N = p.nx * p.ny * p.nz
     st = torch.cuda.current_stream()
@@ -484,7 +486,7 @@ def fp64_alu_roofline(ms_per_step: float, N: int) -> dict:
 
 def _timed(lb, torch, max_over_ranks, barrier, p, rho, T, K, W=10):
     lat = lb.Lattice(p, torch.from_numpy(rho).cuda(), torch.from_numpy(T).cuda())
-    launch = lat.launch_info()
+    launch = lat.step_info()
     lat.step(W)
     torch.cuda.synchronize()
     barrier()
@@ -640,7 +642,7 @@ def variant_sweep(lb, torch, peaks, max_over_ranks, barrier, ws) -> dict:
             rho, T = synthetic.single_phase_fields(p.nx, p.ny, p.nz, 6.0, p.T_d, p.T_u)
         N = p.nx * p.ny * p.nz
         lat = lb.Lattice(p, torch.from_numpy(rho).cuda(), torch.from_numpy(T).cuda())
-        launch = lat.launch_info()
+        launch = lat.step_info()
         lat.step(10)
         torch.cuda.synchronize()
         barrier()

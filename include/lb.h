@@ -245,6 +245,15 @@ long long lb_step_count(const lb_ctx* ctx);
  * per thread. Errors: LB_EINVAL (NULL argument), LB_ECUDA. */
 int lb_launch_info(lb_ctx* ctx, int* out);
 
+/* lb_step_info -- the kernel that a plain step of the context launches (launch metadata; the paper has no
+ * counterpart). Host output of 7 ints: out[0] = form (0 the tile march, 1 three kernels, 2 the march, 3 the
+ * march with two nodes per thread), out[1], out[2] = grid (column tiles, z chunks; three kernels: CTAs per
+ * plane, planes), out[3] = threads per CTA, out[4] = dynamic shared memory bytes per CTA, out[5] = CTAs
+ * resident per SM as the CUDA occupancy calculator reports it, out[6] = registers per thread (three
+ * kernels: out[3] to out[6] of the collision; FP64 tile march: of its second kernel). Errors: LB_EINVAL
+ * (NULL argument), LB_ECUDA. */
+int lb_step_info(lb_ctx* ctx, int* out);
+
 /* lb_free -- release the context and its device memory (synchronises its stream). NULL is a no-op. */
 void lb_free(lb_ctx* ctx);
 

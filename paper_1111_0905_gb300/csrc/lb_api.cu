@@ -386,6 +386,25 @@ int lb_launch_info(lb_ctx* c, int* out) {
   return LB_OK;
 }
 
+int lb_step_info(lb_ctx* c, int* out) {
+  if (!c || !out) return LB_EINVAL;
+  const int var = variant_of(c->p.forcing, c->p.psi_kind);
+  int k[4] = {0, 0, 0, 0};
+  const dim3 grid = fused_grid(c);
+  int form = STEP_TILE, gx = (int)grid.x, gy = (int)grid.y;
+  if (c->form == lb_ctx::kTile) {
+    LB_CU(c, c->ops->info(c->by, var, k));
+  } else {
+    form = c->form == lb_ctx::kThree ? STEP_THREE : (c->march_zc2 > 0 ? STEP_MARCH2 : STEP_MARCH);
+    const int zc = form == STEP_THREE ? 1 : (form == STEP_MARCH2 ? c->march_zc2 : c->march_zc);
+    gx = c->nblk_step; gy = (c->p.nz + zc - 1) / zc;
+    LB_CU(c, c->ops->step_info(form, c->three_nt, var, k));
+  }
+  out[0] = form; out[1] = gx; out[2] = gy;
+  for (int i = 0; i < 4; ++i) out[3 + i] = k[i];
+  return LB_OK;
+}
+
 int lb_init(const lb_params* params, const double* rho_init, const double* T_init,
             int init_on_device, void* cuda_stream, lb_ctx** out) {
   if (!out) return LB_EINVAL;

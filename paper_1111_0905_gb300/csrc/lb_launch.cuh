@@ -19,6 +19,9 @@ inline cudaError_t follow(void (*k)(P...), unsigned grid, int nt, cudaStream_t s
   return cudaLaunchKernelEx(&cfg, k, args...);
 }
 
+// forms of the step as lb_step_info reports them
+enum { STEP_TILE = 0, STEP_THREE = 1, STEP_MARCH = 2, STEP_MARCH2 = 3 };
+
 struct PrecOps {
   size_t esize;        // bytes per stored population
   int deviation;       // 1 if populations are stored as deviations from w_l * ref
@@ -36,6 +39,9 @@ struct PrecOps {
   // one-launch march (lb_march.cuh) with chunks of zc planes and its tile height (0: none for FP64)
   cudaError_t (*split)(const KArgs&, int mode, int nt, cudaStream_t);
   cudaError_t (*march)(const KArgs&, int mode, int zc, int zc2, cudaStream_t);
+  // the kernel of a plain step (three kernels: the collision) of form STEP_* and variant var, CTAs of nt
+  // threads (three kernels only): threads, dynamic shared memory, resident CTAs per SM, registers
+  cudaError_t (*step_info)(int form, int nt, int var, int out[4]);
   int march_ty;
   int march_ty2;       // tile height of the march with two nodes per thread (64 wide; chunks of zc2; 0: none)
   int slots;           // stored slots per lattice and node: 19, or 21 with the local references
@@ -79,20 +85,19 @@ template <class S> struct OpsImpl {
     if ((e = attr_by<16>()) != cudaSuccess) return e;
     return march_prepare();
   }
+  template <class K> static cudaError_t kernel_info(K kernel, int nt, size_t dyn, int out[4]) {
+    cudaFuncAttributes fa;
+    cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
+    if (e != cudaSuccess) return e;
+    int n = 0;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, nt, dyn);
+    if (e != cudaSuccess) return e;
+    out[0] = nt; out[1] = (int)dyn; out[2] = n; out[3] = fa.numRegs;
+    return cudaSuccess;
+  }
   template <int BY, int VAR> static cudaError_t info_var(int out[4]) {
-    if constexpr (!fits<BY>()) {
-      return cudaErrorInvalidConfiguration;
-    } else {
-      cudaFuncAttributes fa;
-      cudaError_t e = cudaFuncGetAttributes(&fa, lb_fused_kernel<S, BY, MODE_STEP, VAR>);
-      if (e != cudaSuccess) return e;
-      int n = 0;
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, lb_fused_kernel<S, BY, MODE_STEP, VAR>,
-                                                        BX * BY, smem<BY>());
-      if (e != cudaSuccess) return e;
-      out[0] = BX * BY; out[1] = (int)smem<BY>(); out[2] = n; out[3] = fa.numRegs;
-      return cudaSuccess;
-    }
+    if constexpr (!fits<BY>()) return cudaErrorInvalidConfiguration;
+    else return kernel_info(lb_fused_kernel<S, BY, MODE_STEP, VAR>, BX * BY, smem<BY>(), out);
   }
   template <int BY> static cudaError_t info_by(int var, int out[4]) {
     switch (var) {
@@ -266,6 +271,30 @@ template <class S> struct OpsImpl {
         case VAR_VDW: return march_go<VAR_VDW, MODE_STEP>(a, b, grid, st);
         default: return march_go<VAR_GUO | VAR_VDW, MODE_STEP>(a, b, grid, st);
       }
+    }
+  }
+  template <int VAR> static cudaError_t step_info_var(int form, int nt, int out[4]) {
+    if (form == STEP_THREE) {
+      if (nt == 32) return kernel_info(split_collide_kernel<S, VAR, MODE_STEP, 32>, 32, 0, out);
+      if (nt == 64) return kernel_info(split_collide_kernel<S, VAR, MODE_STEP, 64>, 64, 0, out);
+      return kernel_info(split_collide_kernel<S, VAR, MODE_STEP, 256>, 256, 0, out);
+    }
+    if constexpr (!std::is_same<S, double>::value) {
+      using GE = MarchGeo<S, MTY>;
+      if (form == STEP_MARCH) return kernel_info(split_march_kernel<S, VAR, MODE_STEP, MTY>, GE::NT, GE::smem, out);
+      if constexpr (MTY2 > 0 && VAR == 0) {
+        using G2 = March2Geo<MTY2>;
+        if (form == STEP_MARCH2) return kernel_info(split_march2_kernel<S, MTY2, false>, G2::NT, G2::smem, out);
+      }
+    }
+    return cudaErrorInvalidValue;
+  }
+  static cudaError_t step_info(int form, int nt, int var, int out[4]) {
+    switch (var) {
+      case 0: return step_info_var<0>(form, nt, out);
+      case VAR_GUO: return step_info_var<VAR_GUO>(form, nt, out);
+      case VAR_VDW: return step_info_var<VAR_VDW>(form, nt, out);
+      default: return step_info_var<VAR_GUO | VAR_VDW>(form, nt, out);
     }
   }
   static int blocks_for(int N) {

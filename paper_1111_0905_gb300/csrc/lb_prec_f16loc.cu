@@ -6,5 +6,5 @@ const PrecOps kOpsF16Loc = {sizeof(half_loc), 1, &OpsImpl<half_loc>::prepare, &O
                     &OpsImpl<half_loc>::init, &OpsImpl<half_loc>::pops,
                     &OpsImpl<half_loc>::tile_ok, &OpsImpl<half_loc>::info,
                     &OpsImpl<half_loc>::setpops, &OpsImpl<half_loc>::split,
-                    &OpsImpl<half_loc>::march, OpsImpl<half_loc>::MTY, OpsImpl<half_loc>::MTY2, slots<half_loc>()};
+                    &OpsImpl<half_loc>::march, &OpsImpl<half_loc>::step_info, OpsImpl<half_loc>::MTY, OpsImpl<half_loc>::MTY2, slots<half_loc>()};
 }  // namespace tlbm

@@ -6,5 +6,5 @@ const PrecOps kOpsF32 = {sizeof(float), 0, &OpsImpl<float>::prepare, &OpsImpl<fl
                     &OpsImpl<float>::init, &OpsImpl<float>::pops,
                     &OpsImpl<float>::tile_ok, &OpsImpl<float>::info,
                     &OpsImpl<float>::setpops, &OpsImpl<float>::split,
-                    &OpsImpl<float>::march, OpsImpl<float>::MTY, OpsImpl<float>::MTY2, slots<float>()};
+                    &OpsImpl<float>::march, &OpsImpl<float>::step_info, OpsImpl<float>::MTY, OpsImpl<float>::MTY2, slots<float>()};
 }  // namespace tlbm

@@ -6,5 +6,5 @@ const PrecOps kOpsF64 = {sizeof(double), 0, &OpsImpl<double>::prepare, &OpsImpl<
                     &OpsImpl<double>::init, &OpsImpl<double>::pops,
                     &OpsImpl<double>::tile_ok, &OpsImpl<double>::info,
                     &OpsImpl<double>::setpops, &OpsImpl<double>::split,
-                    &OpsImpl<double>::march, 0, 0, slots<double>()};
+                    &OpsImpl<double>::march, &OpsImpl<double>::step_info, 0, 0, slots<double>()};
 }  // namespace tlbm

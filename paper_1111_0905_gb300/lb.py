@@ -31,7 +31,8 @@ EXPORTS = ("lb_init", "lb_step", "lb_adjoint_step", "lb_profiles", "lb_histogram
            "lb_structure_functions", "lb_moments", "lb_nusselt", "lb_populations", "lb_diagnostics",
            "lb_save", "lb_load", "lb_step_count", "lb_free", "lb_strerror", "lb_last_error",
            "lb_nusselt_fields_noalloc", "lb_launch_info", "lb_heat_flux_pdf", "lb_set_populations",
-           "lb_stream_bound")
+           "lb_stream_bound", "lb_step_info")
+STEP_FORMS = ("tile march", "three kernels", "march", "march, two nodes per thread")
 NOALLOC_MAX_NZ = 8192
 
 
@@ -142,6 +143,8 @@ def load_library():
     lib.lb_nusselt_fields_noalloc.restype = I
     lib.lb_launch_info.argtypes = [P, P]
     lib.lb_launch_info.restype = I
+    lib.lb_step_info.argtypes = [P, P]
+    lib.lb_step_info.restype = I
     lib.lb_heat_flux_pdf.argtypes = [P, I, I, I, D, D, P, P]
     lib.lb_heat_flux_pdf.restype = I
     lib.lb_stream_bound.argtypes = [I, P, P, P, P, I, I, I, I, ctypes.POINTER(I), P]
@@ -284,11 +287,20 @@ class Lattice:
         return int(self.lib.lb_step_count(self.ctx))
 
     def launch_info(self) -> dict:
-        """lb_launch_info: grid, threads and shared memory per CTA, resident CTAs per SM, registers."""
+        """lb_launch_info: the tile march's grid, threads and shared memory per CTA, resident CTAs per SM,
+        registers (of the kernel that steps: step_info)."""
         out = (ctypes.c_int * 6)()
         self._check(self.lib.lb_launch_info(self.ctx, out), "lb_launch_info")
         return {"grid": [out[0], out[1]], "threads_per_cta": out[2], "smem_bytes": out[3],
                 "ctas_per_sm": out[4], "registers": out[5]}
+
+    def step_info(self) -> dict:
+        """lb_step_info: form, grid, threads and shared memory per CTA, resident CTAs per SM and registers
+        of the kernel that a plain step launches."""
+        out = (ctypes.c_int * 7)()
+        self._check(self.lib.lb_step_info(self.ctx, out), "lb_step_info")
+        return {"form": STEP_FORMS[out[0]], "grid": [out[1], out[2]], "threads_per_cta": out[3],
+                "smem_bytes": out[4], "ctas_per_sm": out[5], "registers": out[6]}
 
     def adjoint(self, nsteps: int, checkpoint_every: int = 50, grad_T0: bool = False) -> dict:
         """lb_adjoint_step: J = time-averaged Nu over the next nsteps steps and dJ/d(T_d, T_u, G)
