@@ -106,7 +106,9 @@ __global__ void histogram_kernel(const double* __restrict__ rho, const double* _
 // Structure functions for horizontal increments: block (r-1, z - z_lo) sums over plane z of
 // (q(x + r e_x) - q(x))^p + (q(x + r e_y) - q(x))^p for q = u_z, T and p = 2, 4. Bound by its 16 FP64
 // instructions per node and r (96^2 x 72 nodes, r <= 32: 0.54 ms at the pipe's rate; 0.66 ms, 0.78
-// before the sums went through shared memory and the rows needed no division).
+// before the sums went through shared memory and the nodes needed no division). Threads take nodes, not
+// rows, so that every lane has one whatever the row length: 33 x 558 x 72 nodes, r <= 31, 1.33 ms a call
+// as for rows of 32 or 96; a warp per row took 3.66, the division per node 1.63.
 __global__ void structure_kernel(const double* __restrict__ uz, const double* __restrict__ T,
                                  int nx, int ny, int z_lo, double* __restrict__ out /* [rmax][nzs][4] */,
                                  int nzs) {
@@ -120,17 +122,18 @@ __global__ void structure_kernel(const double* __restrict__ uz, const double* __
     s2 += p; s2 += q;
     s4 = fma(p, p, s4); s4 = fma(q, q, s4);
   };
-  // a warp per row, its lanes along x
-  for (int y = (int)(threadIdx.x >> 5); y < ny; y += kWarps) {
-    const int yr = y + r < ny ? y + r : y + r - ny;
-    const double *u0 = uz + base + (size_t)y * nx, *ur = uz + base + (size_t)yr * nx;
-    const double *t0 = T + base + (size_t)y * nx, *tr = T + base + (size_t)yr * nx;
-    for (int x = (int)(threadIdx.x & 31); x < nx; x += 32) {
-      const int xr = x + r < nx ? x + r : x + r - nx;
-      const double u = u0[x], t = t0[x];
-      take(u0[xr] - u, ur[x] - u, a2, a4);
-      take(t0[xr] - t, tr[x] - t, b2, b4);
-    }
+  // node by node over the plane, its column and row carried along
+  const int nxy = nx * ny, dx = kThreads % nx, dy = kThreads / nx;
+  int x = (int)threadIdx.x % nx, y = (int)threadIdx.x / nx;
+  const double *up = uz + base, *tp = T + base;
+  for (int k = (int)threadIdx.x; k < nxy; k += kThreads) {
+    const int kx = x + r < nx ? k + r : k + r - nx;
+    const int ky = y + r < ny ? k + r * nx : k + (r - ny) * nx;
+    const double u = up[k], t = tp[k];
+    take(up[kx] - u, up[ky] - u, a2, a4);
+    take(tp[kx] - t, tp[ky] - t, b2, b4);
+    x += dx; y += dy;
+    if (x >= nx) { x -= nx; ++y; }
   }
   const double v[4] = {a2, a4, b2, b4};
   const double s = block_sum4(v, sh);
