@@ -152,10 +152,9 @@ KArgs make_args(const lb_ctx* c) {
     a.fd_rho = next(); a.fd_psi = next();
     for (int k = 0; k < 3; ++k) a.fd_j[k] = next();
     for (int k = 0; k < 3; ++k) a.fd_u[k] = next();
-    if (f64) {
-      for (int k = 0; k < 3; ++k) a.fd_v[k] = next();
-      a.fd_inv = next();
-    }
+    // FP32: u' takes the place of j, which its own node has read by then (16-bit storage keeps none)
+    for (int k = 0; k < 3; ++k) a.fd_v[k] = f64 ? next() : (c->ops->esize == 4 ? a.fd_j[k] : nullptr);
+    if (f64) a.fd_inv = next();
   }
   // i / nx by multiplication, exact for i < 2^31: m = ceil(2^(32+s) / nx), 2^s < nx <= 2^(s+1)
   if (c->p.nx > 1) {
@@ -248,8 +247,8 @@ namespace {
 // start, one CTA per SM, in waves: ceil(CTAs / SMs) (zc + 6) iterations. Measured per iteration (128^3,
 // 256^3): FP32 1.8 us, 16-bit deviations 1.5 us (two nodes per thread: 2.2 us for a tile of twice the
 // width, 7 rows), local references 2.2 us. The three kernels take about
-// 7 us and per node 73, 58 and 77 ps (FP32 64^3 28 us and 128^3 168 us, the march 21 and 126 us; 32^3
-// 7.6 us against 18; local references 96^3 72 us against 86). The chunk zc is the one of the least cost.
+// 7 us and per node 75, 58 and 77 ps (FP32 64^3 28 us and 128^3 172 us, the march 21 and 126 us; 32^3
+// 7.4 us against 18; local references 96^3 72 us against 86). The chunk zc is the one of the least cost.
 cudaError_t choose_form(lb_ctx* c) {
   c->nblk = c->nblk_step = c->ntiles;
   if (c->p.tile_y != 0 || c->p.z_chunk != 0) { c->form = lb_ctx::kTile; return cudaSuccess; }
@@ -275,7 +274,7 @@ cudaError_t choose_form(lb_ctx* c) {
     const long long tiles = (long long)c->tiles_x * rows(c->ops->march_ty);
     const long long best = chunk(tiles, &c->march_zc);
     const bool b16 = c->ops->esize == 2, loc = c->ops->slots > Q;
-    const double node = loc ? 77e-12 : (b16 ? 58e-12 : 73e-12);
+    const double node = loc ? 77e-12 : (b16 ? 58e-12 : 75e-12);
     double march = (loc ? 2.2e-6 : (b16 ? 1.5e-6 : 1.8e-6)) * (double)best;
     const long long tiles2 = c->ops->march_ty2 > 0 ? (long long)((c->p.nx + 63) / 64) * rows(c->ops->march_ty2) : 0;
     if (tiles2 > 0 && c->p.nx % 2 == 0 && variant_of(c->p.forcing, c->p.psi_kind) == 0) {

@@ -1,12 +1,12 @@
 // lb_split.cuh -- the time step as three streaming kernels, one node per thread:
 //
 //   moments   pull f; write rho (FP32 compute: drho; FP64: and 1/rho), j and psi;
-//   velocity  gather psi (Eq. (9)); write the physical velocity u = (j + F/2)/rho (FP64: and the
-//             equilibrium velocity u' = (j + tau F)/rho; Guo forcing: F in its place);
+//   velocity  gather psi (Eq. (9)); write the physical velocity u = (j + F/2)/rho and, but for 16-bit
+//             storage, the equilibrium velocity u' = (j + tau F)/rho (Guo forcing: F in its place);
 //   collide   pull f and g, div(u) from six neighbours, collide and write both lattices.
 //
-// Per node FP32 moves 76 + 16, 20 + 12 and 152 + 16 + 152 bytes in them, each at about the rate of a
-// copy (256^3: 0.23, 0.15 and 0.84 ms); FP64 executes 61, 35 and 187 FP64 instructions, each at the rate
+// Per node FP32 moves 76 + 20, 20 + 24 and 152 + 28 + 152 bytes in them, at about the rate of a copy (161 x
+// 210 x 128: 328 us); FP64 executes 61, 35 and 187 FP64 instructions, each at the rate
 // of the FP64 pipe (128^3: 245, 139 and 735 us; the tile march with its pre-pass 1543).
 // Nothing is recomputed and nothing waits at a barrier: the form of the FP64 step, which its FP64
 // instructions bound, and of the cells too small to fill the GPU with marching CTAs, where the
@@ -363,10 +363,9 @@ __global__ void __launch_bounds__(NT) split_velocity_kernel(const KArgs a, int n
   for (int k = 0; k < 3; ++k) {
     const R ji = j[k] * inv;
     st_at(static_cast<R*>(a.fd_u[k]) + zo, n.i, mu * A[k] + (k == 2 ? ji + kp.gz_u : ji));
-    if constexpr (F64) {
-      if constexpr (GUO) st_at(static_cast<R*>(a.fd_v[k]) + zo, n.i, k == 2 ? mg * A[k] + rho * kp.g_z : mg * A[k]);
-      else st_at(static_cast<R*>(a.fd_v[k]) + zo, n.i, mv * A[k] + (k == 2 ? ji + kp.gz_v : ji));
-    }
+    if (!F64 && a.fd_v[k] == nullptr) continue;       // 16-bit storage
+    if constexpr (GUO) st_at(static_cast<R*>(a.fd_v[k]) + zo, n.i, k == 2 ? mg * A[k] + rho * kp.g_z : mg * A[k]);
+    else st_at(static_cast<R*>(a.fd_v[k]) + zo, n.i, mv * A[k] + (k == 2 ? ji + kp.gz_v : ji));
   }
   if constexpr (F64) {
     if (a.adj_m != nullptr) {
@@ -439,10 +438,11 @@ __global__ void __launch_bounds__(NT, split_mb<S, MODE>() * 256 / NT) split_coll
       // 2 div(u)
       const R D2 = ((ld_at(pux, xs[2] + ys[1]) - ld_at(pux, xs[0] + ys[1])) +
                     (ld_at(puy, xs[1] + ys[2]) - ld_at(puy, xs[1] + ys[0]))) + (uzp - uzm);
-      // u' (Guo forcing: F). FP32 compute: from u = (j + F/2)/rho and j of the pulled f, which saves
-      // writing and reading three fields; FP64 reads them (its FP64 instructions cost more)
+      // u' (Guo forcing: F) as the velocity pass formed it. 16-bit storage: from u = (j + F/2)/rho and j
+      // of the pulled f, which saves writing and reading three fields (6 % of a step). That costs
+      // 2^-24 |u| of F tau/rho; its populations are rounded to 2^-12, FP32's are not.
       R w[3];
-      if constexpr (F64) {
+      if constexpr (sizeof(S) != 2) {
 #pragma unroll
         for (int k = 0; k < 3; ++k) w[k] = ld_at(static_cast<const R*>(a.fd_v[k]) + zo, o);
       } else {
