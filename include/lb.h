@@ -61,7 +61,8 @@ typedef enum {
  * not over long boiling runs (4e-2 after 5000 steps: the phase pattern drifts); bfloat16 deviations
  * only over a few tens of steps (within 2e-3 after 50 steps of a 32^3 cell, 3.8e-3 after 100 steps
  * of the 512^3 boiling cell); float16 against local references within 2e-3 over both horizons
- * (2.3e-4 after 5000 boiling steps of the 256^3 cell). */
+ * (2.6e-4 after 5000 boiling steps of the 256^3 cell). FP32 compute relaxes at 1 - r, r = 1 - 1/tau
+ * rounded to float32: within 3e-8 of 1/tau, exactly at tau = 1. */
 
 /* Scheme variants for comparison with the paper's scheme (variant 0 of each; the paper defines
  * neither alternative). Forcing: LB_FORCE_SHIFT, the paper's equilibrium velocity
@@ -115,8 +116,8 @@ int lb_init(const lb_params* params, const double* rho_init, const double* T_ini
 
 /* lb_step -- advance nsteps time steps of Eqs. (6)-(7). A context with a launch shape (tile_y or
  * z_chunk) takes the tile march: per step one fused launch (FP64: after a pass that forms the moments
- * of every node). Otherwise the library chooses by precision and grid size between a march in one
- * launch with separate warps for the moments and the collision, and three streaming kernels
+ * of every node). Otherwise the library chooses by precision, grid size and the device's SMs between a
+ * march in one launch with separate warps for the moments and the collision, and three streaming kernels
  * (moments, velocities, collision); the forms differ in rounding only. In the forms that it chooses a
  * step that takes a Nu sample (nu_every) and one that does not leave the same populations, bit for bit,
  * and so do runs with lb_nusselt, lb_diagnostics, lb_save or lb_load between their steps. A step
@@ -239,9 +240,9 @@ long long lb_step_count(const lb_ctx* ctx);
 
 /* lb_launch_info -- the launch shape of the context's tile march, the step kernel of a context with
  * tile_y or z_chunk set (a context that leaves both 0 steps with the form that lb_step describes);
- * launch metadata for performance reports, the paper has no counterpart. Host output of 6 ints: out[0], out[1] = grid (column
- * tiles, z chunks), out[2] = threads per CTA, out[3] = dynamic shared memory bytes per CTA,
- * out[4] = CTAs resident per SM as the CUDA occupancy calculator reports it, out[5] = registers
+ * launch metadata for performance reports, the paper has no counterpart. Host output of 6 ints: out[0],
+ * out[1] = grid (column tiles, z chunks), out[2] = threads per CTA, out[3] = dynamic shared memory bytes
+ * per CTA, out[4] = CTAs resident per SM as the CUDA occupancy calculator reports it, out[5] = registers
  * per thread. Errors: LB_EINVAL (NULL argument), LB_ECUDA. */
 int lb_launch_info(lb_ctx* ctx, int* out);
 

@@ -236,9 +236,8 @@ extern "C" int lb_profiles(lb_ctx* c, double* rho_z, double* T_z, double* PdivU_
   const size_t n = (size_t)3 * nz * np;
   if (cudaMalloc(&out.p, n * sizeof(double)) != cudaSuccess) return lb_fail(c, LB_ENOMEM, "profiles");
   ana::profiles_kernel<<<(unsigned)np * (unsigned)nz, ana::kThreads, 0, c->stream>>>(
-      np,rho, ux, uy, uz, T, c->p.nx, c->p.ny, nz, c->p.G,
-                                                  c->p.psi_kind, c->p.vdw_a, c->p.vdw_b, c->p.vdw_T,
-                                                  static_cast<double*>(out.p));
+      np, rho, ux, uy, uz, T, c->p.nx, c->p.ny, nz, c->p.G, c->p.psi_kind, c->p.vdw_a, c->p.vdw_b, c->p.vdw_T,
+      static_cast<double*>(out.p));
   LB_CU(c, cudaGetLastError());
   std::vector<double> h(n);
   LB_CU(c, cudaMemcpyAsync(h.data(), out.p, h.size() * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
@@ -289,8 +288,8 @@ extern "C" int lb_structure_functions(lb_ctx* c, int rmax, int z_lo, int z_hi, d
   DevBuf out;
   const size_t n = (size_t)rmax * nzs * 4;
   if (cudaMalloc(&out.p, n * sizeof(double)) != cudaSuccess) return lb_fail(c, LB_ENOMEM, "structure functions");
-  ana::structure_kernel<<<dim3(rmax, nzs), ana::kThreads, 0, c->stream>>>(uz, T, c->p.nx, c->p.ny, z_lo,
-                                                                static_cast<double*>(out.p), nzs);
+  ana::structure_kernel<<<dim3(rmax, nzs), ana::kThreads, 0, c->stream>>>(
+      uz, T, c->p.nx, c->p.ny, z_lo, static_cast<double*>(out.p), nzs);
   LB_CU(c, cudaGetLastError());
   std::vector<double> h(n);
   LB_CU(c, cudaMemcpyAsync(h.data(), out.p, n * sizeof(double), cudaMemcpyDeviceToHost, c->stream));

@@ -2,7 +2,8 @@
 //
 // Host side: parameter validation, device memory of the context (two ping-pong population
 // lattices per distribution, diagnostics scratch), launch geometry, checkpoints. Every step of
-// the method runs in the kernels of lb_kernels.cuh; this file only marshals and orders them.
+// the method runs in the kernels of lb_kernels.cuh, lb_split.cuh, lb_march.cuh and lb_march2.cuh; this
+// file chooses the form of the step and marshals and orders them.
 #include <cuda_runtime.h>
 
 #include <algorithm>

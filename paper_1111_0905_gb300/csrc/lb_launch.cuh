@@ -1,4 +1,5 @@
-// lb_launch.cuh -- per-precision launch table of the kernels in lb_kernels.cuh.
+// lb_launch.cuh -- per-precision launch table of the kernels in lb_kernels.cuh, lb_split.cuh, lb_march.cuh
+// and lb_march2.cuh.
 // Each precision is compiled in its own translation unit (lb_prec_*.cu) that defines one table.
 #pragma once
 #include "lb_kernels.cuh"

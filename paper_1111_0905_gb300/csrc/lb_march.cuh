@@ -10,10 +10,10 @@
 //
 // Why two groups: the tile march (lb_kernels.cuh) runs its stages one after the other in the same 16
 // warps, each blocked on its own loads; here every load is requested a plane before its use and the
-// stages of different planes overlap. FP32 256^3 boiling cell 1.279 -> 0.948 ms a step, 5.4 TB/s of DRAM
-// traffic (81 % of a copy), 512^3 9.88 -> 7.45 ms, 128^3 184 -> 126 us; leaving out any of its loads or
+// stages of different planes overlap. FP32 256^3 boiling cell 1.279 -> 0.944 ms a step, 5.4 TB/s of DRAM
+// traffic (81 % of a copy), 512^3 9.88 -> 7.57 ms, 128^3 184 -> 126 us; leaving out any of its loads or
 // stores shortens it by the bytes' share: memory traffic bounds it. 16-bit storage: instructions (issue
-// slots 59-70 % busy); local references 256^3 1.544 -> 1.174 ms.
+// slots 59-70 % busy); local references 256^3 1.544 -> 1.19 ms.
 #pragma once
 #include "lb_split.cuh"
 
