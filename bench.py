@@ -44,7 +44,7 @@ STORED_SLOTS = {"f64": 19, "f32": 19, "bf16dev": 19, "fp16dev": 19, "fp16loc": 2
 PATTERN_FORMS = ("f32", "fp16dev", "bf16dev")
 # the kernel that takes most of a step of the headline cell
 STEP_KERNEL = {"f64": "split_collide_kernel<double,0,0,256>", "f32": "split_march_kernel<float,0,0,8>",
-               "bf16dev": "split_march2_kernel<__nv_bfloat16,7>", "fp16dev": "split_march2_kernel<__half,7>",
+               "bf16dev": "split_march2_kernel<__nv_bfloat16,7,0>", "fp16dev": "split_march2_kernel<__half,7,0>",
                "fp16loc": "split_march_kernel<tlbm::half_loc,0,0,7>"}
 
 # DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) per launch of the fused step
@@ -52,9 +52,9 @@ STEP_KERNEL = {"f64": "split_collide_kernel<double,0,0,256>", "f32": "split_marc
 # launch time is kept to a few GB on the device), keyed by the hash of the kernel sources it
 # was taken on. The headline's traffic is that capture scaled by the node count (the traffic
 # of one launch grows in proportion to the nodes it updates); null once the sources changed.
-TRAFFIC = {"src_hash": "a6c6f191f804461b", "nodes": 256 ** 3,
-           "bytes_per_launch": {"f32": 2659395584 + 2508636160, "fp16loc": 1455475456 + 1370433024,
-                                "fp16dev": 1294676224 + 1226098944},
+TRAFFIC = {"src_hash": "9d68a38fe0c72ba2", "nodes": 256 ** 3,
+           "bytes_per_launch": {"f32": 2647133952 + 2507949568, "fp16loc": 1447681024 + 1369994240,
+                                "fp16dev": 1293137664 + 1226472704},
            "what": "ncu DRAM bytes of one launch of the 256^3 paper-geometry cell, scaled by the node count"}
 
 # FP64 operations per node of one FP64 step (ncu: 2 x DFMA + DADD + DMUL thread instructions of the

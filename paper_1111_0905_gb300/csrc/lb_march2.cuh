@@ -5,8 +5,8 @@
 // without an x shift are pulled, kept and stored as 4-byte words, psi and the velocities are read and
 // written in pairs, and a 64-wide tile recomputes fewer ring nodes. For even nx (a pair never crosses
 // the periodic edge and every word is aligned) and the paper's scheme; everything else takes the one-node
-// march. 867 instructions a node; FP16 256^3 boiling cell 722 -> 608 us a step, 512^3 5.58 -> 4.88 ms,
-// 128^3 105 -> 84 us.
+// march. 869 instructions a node; FP16 256^3 boiling cell 722 -> 613 us a step, 512^3 5.58 -> 4.92 ms,
+// 128^3 105 -> 86 us.
 #pragma once
 #include "lb_march.cuh"
 
